@@ -13,7 +13,7 @@ CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 OUT = os.path.join(HERE, "_lib", "libmatcha.so")
 PROBE = os.path.join(HERE, "_lib", "libpeakprobe.so")
-SOURCES = ["matcha_api.cu", "plan_tables.cu", "analyze.cu", "correlate.cu", "soft.cu", "newton.cu",
+SOURCES = ["matcha_api.cu", "plan_tables.cu", "analyze.cu", "correlate.cu", "soft.cu", "soft_grid.cu", "newton.cu",
            "noalloc.cu", "backward.cu", "translate.cu", "pose6d.cu", "ball.cu",
            "correlate_tc.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]

@@ -60,6 +60,7 @@ struct Plan {
   void *phi_cs;                 // real [np][2]: cos, sin (2 pi k / n_phi)
   void *soft_tw;                // real [ns][2]: cos, sin (2 pi t / ns)
   void *soft_d;                 // real [ns][nc0]: d^l_mn(beta_k) in the SOFFT layout
+  void *soft_dT;                // real [nc0][ns]: soft_d transposed
   void *rcoef;                  // real, grouped layout: (a, -b, -e) of the step l -> l+1, -l(l+1)
   void *seedK;                  // real [ngroups][4]: (sqrt(binom(2m, m+n)) of both halves, 0, 0)
   void *dft_cs;                 // real [2][2][Qf][Mq]: folded phi-DFT table (parity, cos|sin, q, column)
@@ -163,6 +164,9 @@ bool correlate_tc_fits(int S, int L, int bytes);
 bool backward_fits(const Plan &p);  // the template-gradient kernel's shared memory fits
 bool newton_fits(const Plan &p);  // the refinement kernel's shared memory fits
 bool analyze_shells_ok(const Plan &p, int G);  // G shells per analysis CTA fit
+template <typename T>  // the search through memory (soft_grid.cu)
+cudaError_t launch_soft_grid(const Plan &p, const T *c, int B, const int *P_per, T *grid, int *idx,
+                             double *euler, double *score, int *n_cand, cudaStream_t st);
 bool soft_grid_optional(const Plan &p);  // the SOFFT search can skip writing the grid
 bool soft_fits(const Plan &p);           // some SOFFT kernel serves the plan
 bool soft_warps_ok(const Plan &p);       // the warp-per-slice SOFFT kernel serves the plan

@@ -188,7 +188,7 @@ matcha_status matcha_plan_create(const matcha_plan_desc *d, matcha_plan *out) {
   auto add = [&](size_t bytes) { size_t o = sz; sz = align_up(sz + bytes); return o; };
   size_t o_rs = add(8 * p->S), o_w = add(8 * p->S), o_x = add(8 * p->nt), o_wj = add(8 * p->nt);
   size_t o_pt = add(rs * p->nlm * p->nt), o_phi = add(rs * 2 * p->np), o_tw = add(rs * 2 * p->ns);
-  size_t o_sd = add(rs * p->ns * p->nc0), o_rc = add(rs * 4 * p->nc), o_K = add(rs * 4 * p->ngroups);
+  size_t o_sd = add(rs * p->ns * p->nc0), o_sdT = add(rs * p->ns * p->nc0), o_rc = add(rs * 4 * p->nc), o_K = add(rs * 4 * p->ngroups);
   size_t o_off = add(4 * p->npairs), o_off0 = add(4 * p->npairs0);
   size_t o_ptl = add(rs * p->nlm * p->nt), o_leg = add(4 * (size_t)p->nlm);
   size_t o_dcs = add(rs * 4 * (size_t)p->Qf * p->Mq);
@@ -202,7 +202,7 @@ matcha_status matcha_plan_create(const matcha_plan_desc *d, matcha_plan *out) {
   char *b = (char *)p->base;
   p->rs = (double *)(b + o_rs); p->wrad = (double *)(b + o_w);
   p->xj = (double *)(b + o_x); p->wj = (double *)(b + o_wj);
-  p->ptab = b + o_pt; p->phi_cs = b + o_phi; p->soft_tw = b + o_tw; p->soft_d = b + o_sd;
+  p->ptab = b + o_pt; p->phi_cs = b + o_phi; p->soft_tw = b + o_tw; p->soft_d = b + o_sd; p->soft_dT = b + o_sdT;
   p->rcoef = b + o_rc; p->seedK = b + o_K;
   p->pair_base = (int *)(b + o_off); p->pair_off0 = (int *)(b + o_off0);
   p->ptab_leg = b + o_ptl; p->leg_lm = (int *)(b + o_leg);

@@ -206,6 +206,14 @@ __global__ void k_ptab_leg(int nt, int nlm, const int *leg, const T *in, T *out)
   out[t] = in[(long)j * nlm + l * (l + 1) / 2 + m];
 }
 
+// out[e][k] = in[k][e] for ns x n tables.
+template <typename T>
+__global__ void k_transpose(int ns, long n, const T *in, T *out) {
+  const long t = blockIdx.x * (long)blockDim.x + threadIdx.x;
+  if (t >= n * ns) return;
+  out[t] = in[(t % ns) * n + t / ns];
+}
+
 cudaError_t build_tables(Plan &p, cudaStream_t st) {
   // scratch for the FP64 versions of the real tables
   size_t n_ptab = (size_t)p.nlm * p.nt, n_phi = 2 * (size_t)p.np, n_tw = 2 * (size_t)p.ns;
@@ -247,6 +255,13 @@ cudaError_t build_tables(Plan &p, cudaStream_t st) {
         {dcs, p.dft_cs, n_dcs}, {ring, p.ring, n_ring}};
     for (auto &c : cp)
       k_to_float<<<(unsigned)((c.n + 255) / 256), 256, 0, st>>>(c.src, (float *)c.dst, (long)c.n);
+  }
+  {
+    const unsigned nb = (unsigned)((n_softd + 255) / 256);
+    if (p.fp64)
+      k_transpose<double><<<nb, 256, 0, st>>>(p.ns, p.nc0, (const double *)p.soft_d, (double *)p.soft_dT);
+    else
+      k_transpose<float><<<nb, 256, 0, st>>>(p.ns, p.nc0, (const float *)p.soft_d, (float *)p.soft_dT);
   }
   {
     const unsigned nb = (unsigned)((n_ptab + 255) / 256);
