@@ -9,6 +9,9 @@
 
 namespace matcha {
 
+// Reals of a partner group's refinement descriptor (layout: k_group_desc).
+constexpr int GROUP_DESC = 40;
+
 // Texture views of a batch of volumes for the analysis gathers: 2-D
 // pitch-linear views (x, z N + y) of runs of `vpt` consecutive volumes, so
 // one 2x2 texture gather fetches the four x-y corners of a trilinear cell in
@@ -36,6 +39,7 @@ struct Plan {
   int refine;    // 0 Newton steps, 1 gradient steps
   int tc;        // contraction on the tensor cores: 0 no, 1 TF32, 2 BF16 (FP32 plans)
   int *dev_err;  // device word: bit 0 = a tensor-core wait reached its limit
+  int sms = 1;                     // SMs of that device
   int device = -1;                 // the CUDA device current at plan creation
   void *noalloc_grid = nullptr;    // device address of the allocation-free search's array
   // tile choices set by matcha_plan_autotune (0 = the built-in rule); none of
@@ -63,6 +67,9 @@ struct Plan {
   void *soft_dT;                // real [nc0][ns]: soft_d transposed
   void *rcoef;                  // real, grouped layout: (a, -b, -e) of the step l -> l+1, -l(l+1)
   void *seedK;                  // real [ngroups][4]: (sqrt(binom(2m, m+n)) of both halves, 0, 0)
+  void *gdesc;                  // real [ngroups][GROUP_DESC]: refinement constants of each group
+  int4 *sched;                  // [sub-slot][nrounds]: newton_schedule
+  int nrounds;
   void *dft_cs;                 // real [2][2][Qf][Mq]: folded phi-DFT table (parity, cos|sin, q, column)
   int Mp;                       // analysis F row: orders padded to a multiple of 4, plus 1
   int Qf, Mq;                   // folded DFT rows ceil(L_J/2); columns per order parity, padded to 4
@@ -162,6 +169,16 @@ cudaError_t launch_correlate_tc(const Plan &p, const float *f, const float *h, i
                                 float *c, cudaStream_t st);
 bool correlate_tc_fits(int S, int L, int bytes);
 bool backward_fits(const Plan &p);  // the template-gradient kernel's shared memory fits
+int newton_slots(const Plan &p);                  // sub-slots of a particle's sums
+size_t newton_smem(const Plan &p);                // of one CTA per particle
+bool newton_rescaled(const Plan &p);              // the rescaled 32-bit recurrence runs
+int newton_schedule(const Plan &p, std::vector<int4> &out);  // returns the rounds
+template <typename T>  // false: not launched, one CTA per particle is as fast
+bool launch_newton_spread(const Plan &p, const T *c, int B, const int *n_cand, double *euler,
+                          double *score, int *cflags, long long *work, cudaStream_t st, cudaError_t *e);
+template <typename T>
+bool launch_objective_spread(const Plan &p, const T *c, int B, int L, int Q, const double *pts,
+                             double *out, cudaStream_t st, cudaError_t *e);
 bool newton_fits(const Plan &p);  // the refinement kernel's shared memory fits
 bool analyze_shells_ok(const Plan &p, int G);  // G shells per analysis CTA fit
 template <typename T>  // the search through memory (soft_grid.cu)

@@ -195,8 +195,14 @@ matcha_status matcha_plan_create(const matcha_plan_desc *d, matcha_plan *out) {
   size_t o_ring = add(rs * 2 * (size_t)p->S * p->nt);
   size_t o_err = add(sizeof(int));
   size_t o_fft = add(rs * 2 * (size_t)p->N);
+  size_t o_gd = add(rs * GROUP_DESC * (size_t)p->ngroups);
+  std::vector<int4> sched;
+  p->nrounds = newton_schedule(*p, sched);
+  size_t o_sch = add(sizeof(int4) * sched.size());
   cudaError_t e = cudaGetDevice(&p->device);
   if (e != cudaSuccess) { delete p; return fail_cuda(e, "cudaGetDevice"); }
+  cudaDeviceGetAttribute(&p->sms, cudaDevAttrMultiProcessorCount, p->device);
+  if (p->sms <= 0) p->sms = 1;
   e = cudaMalloc(&p->base, sz);
   if (e != cudaSuccess) { delete p; return fail_cuda(e, "cudaMalloc(plan tables)"); }
   char *b = (char *)p->base;
@@ -210,6 +216,8 @@ matcha_status matcha_plan_create(const matcha_plan_desc *d, matcha_plan *out) {
   p->ring = b + o_ring;
   p->dev_err = (int *)(b + o_err);
   p->fft_tw = b + o_fft;
+  p->gdesc = b + o_gd;
+  p->sched = (int4 *)(b + o_sch);
   {  // radices of the box FFT (translation search): 4s first, then 2, 3, 5
     int n = p->N, np = 0;
     while (n % 4 == 0 && np < 16) { p->fft_radix[np++] = 4; n /= 4; }
@@ -228,6 +236,8 @@ matcha_status matcha_plan_create(const matcha_plan_desc *d, matcha_plan *out) {
   if (e == cudaSuccess)
     e = cudaMemcpy(p->fft_tw, p->fp64 ? (const void *)tw.data() : (const void *)twf.data(),
                    rs * 2 * (size_t)p->N, cudaMemcpyHostToDevice);
+  if (e == cudaSuccess)
+    e = cudaMemcpy(p->sched, sched.data(), sizeof(int4) * sched.size(), cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemcpy(p->pair_base, base.data(), 4 * p->npairs, cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemcpy(p->pair_off0, off0.data(), 4 * p->npairs0, cudaMemcpyHostToDevice);
   {  // Legendre items: m ascending, then the parity of l + m, then l

@@ -39,16 +39,13 @@
 //   acceptance test and the scores are FP64 in every plan; the 3x3 solve is
 //   FP64 on the final level and in the plan's precision (FP32 for the 32-bit
 //   plans) on the earlier levels.
-#include <math.h>
 #include <algorithm>
-#include "internal.cuh"
+#include "newton_common.cuh"
 
 namespace matcha {
 
 constexpr int NEWTON_THREADS = 256;
 constexpr int NEWTON_WARPS = NEWTON_THREADS / 32;
-
-enum { ST_RUN = 0, ST_TRIAL = 1, ST_STOP = 2, ST_DEAD = 3 };
 
 struct NewtonArgs {
   int LJ, nlev, M, P, cpw, nslots;
@@ -58,24 +55,6 @@ struct NewtonArgs {
   long nc;
 };
 
-template <typename T>
-__device__ __forceinline__ T ipow_t(T x, int e) {
-  T r = T(1);
-  while (e) {
-    if (e & 1) r *= x;
-    x *= x;
-    e >>= 1;
-  }
-  return r;
-}
-
-template <typename T> __device__ __forceinline__ T tcos(T x);
-template <typename T> __device__ __forceinline__ T tsin(T x);
-template <> __device__ __forceinline__ float tcos<float>(float x) { return cosf(x); }
-template <> __device__ __forceinline__ float tsin<float>(float x) { return sinf(x); }
-template <> __device__ __forceinline__ double tcos<double>(double x) { return cos(x); }
-template <> __device__ __forceinline__ double tsin<double>(double x) { return sin(x); }
-
 struct SmemLayout {
   double *th, *tr, *del, *Cc, *res;
   void *red;  // [warps][P][10] working precision
@@ -83,76 +62,9 @@ struct SmemLayout {
   void *ea, *pw, *stage;
 };
 
-// Asynchronous global -> shared copies (no registers involved).
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::); }
-template <int N> __device__ __forceinline__ void cp_async_wait() {
-  asm volatile("cp.async.wait_group %0;\n" ::"n"(N));
-}
-
-// Shared-memory addressing: the hot loops address shared memory through
-// 32-bit shared-window addresses and ld.shared, so every load is a shared
-// load with 32-bit address arithmetic.
-__device__ __forceinline__ unsigned smem_u32(const void *p) {
-  return (unsigned)__cvta_generic_to_shared(p);
-}
 __device__ __forceinline__ void cp_async16s(unsigned sa, const void *gmem) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 16;\n" ::"r"(sa), "l"(gmem));
 }
-__device__ __forceinline__ void lds1(unsigned a, float &x) {
-  asm volatile("ld.shared.f32 %0, [%1];\n" : "=f"(x) : "r"(a));
-}
-__device__ __forceinline__ void lds1(unsigned a, double &x) {
-  asm volatile("ld.shared.f64 %0, [%1];\n" : "=d"(x) : "r"(a));
-}
-__device__ __forceinline__ void lds2(unsigned a, float2 &v) {
-  asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];\n" : "=f"(v.x), "=f"(v.y) : "r"(a));
-}
-__device__ __forceinline__ void lds2(unsigned a, double2 &v) {
-  asm volatile("ld.shared.v2.f64 {%0, %1}, [%2];\n" : "=d"(v.x), "=d"(v.y) : "r"(a));
-}
-// two pairs: 16 bytes in FP32 (one vector load), 32 bytes in FP64
-__device__ __forceinline__ void lds4(unsigned a, float2 &lo, float2 &hi) {
-  asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];\n"
-               : "=f"(lo.x), "=f"(lo.y), "=f"(hi.x), "=f"(hi.y)
-               : "r"(a));
-}
-__device__ __forceinline__ void lds4(unsigned a, double2 &lo, double2 &hi) {
-  lds2(a, lo);
-  lds2(a + 16, hi);
-}
-
-// Two-wide values: the two halves of a partner group (pairs (m, n) and
-// (m, n+1)) advance together.  FP32 uses the packed FP32x2 instructions of the
-// sm_100 family (one FFMA2 does both halves); FP64 issues two scalar FMAs.
-template <typename T> struct Vec2;
-template <> struct Vec2<float> { using type = float2; };
-template <> struct Vec2<double> { using type = double2; };
-template <typename T> using v2 = typename Vec2<T>::type;
-
-__device__ __forceinline__ float2 vfma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
-__device__ __forceinline__ float2 vmul(float2 a, float2 b) { return __fmul2_rn(a, b); }
-__device__ __forceinline__ float2 vadd(float2 a, float2 b) { return __fadd2_rn(a, b); }
-__device__ __forceinline__ double2 vfma(double2 a, double2 b, double2 c) {
-  return make_double2(fma(a.x, b.x, c.x), fma(a.y, b.y, c.y));
-}
-__device__ __forceinline__ double2 vmul(double2 a, double2 b) {
-  return make_double2(a.x * b.x, a.y * b.y);
-}
-__device__ __forceinline__ double2 vadd(double2 a, double2 b) {
-  return make_double2(a.x + b.x, a.y + b.y);
-}
-template <typename T> __device__ __forceinline__ v2<T> vset(T x, T y);
-template <> __device__ __forceinline__ float2 vset<float>(float x, float y) { return make_float2(x, y); }
-template <> __device__ __forceinline__ double2 vset<double>(double x, double y) {
-  return make_double2(x, y);
-}
-template <typename T> __device__ __forceinline__ v2<T> vld(unsigned a0, unsigned a1) {
-  T x, y;
-  lds1(a0, x);
-  lds1(a1, y);
-  return vset<T>(x, y);
-}
-
 struct Group {
   int m, na, off;  // order, first partner's n, offset in (group, l) entries
 };
@@ -182,17 +94,6 @@ struct GroupWalk {
 constexpr int STAGE_BATCH = 4;
 constexpr int STAGE_HDR = 8 * STAGE_BATCH;  // reals
 __host__ __device__ __forceinline__ int stage_half(int LJ) { return STAGE_HDR + 16 * (LJ + 1); }
-
-// Per-candidate tables, candidate index fastest with an odd stride
-// cand_stride(P) >= P, so the lanes of a sub-slot (one candidate each) read
-// distinct banks.  Power table: two rows (cos(b/2)^k, sin(b/2)^k), each
-// PW_PAD zeros followed by k = 0 .. 2 L_J + 3.  Phase table: four rows
-// (cos k a, sin k a, cos k g, sin k g) for k = -L_J .. L_J + 1 (index k + L_J).
-// Element (row r, position k, candidate p) is at (r * row_len + k) * stride + p.
-constexpr int PW_PAD = 4;
-__host__ __device__ __forceinline__ int pw_row(int LJ) { return PW_PAD + 2 * LJ + 4; }
-__host__ __device__ __forceinline__ int ph_row(int LJ) { return 2 * LJ + 2; }
-__host__ __device__ __forceinline__ int cand_stride(int P) { return P | 1; }
 
 // Seeds at l = m of both halves: d = sigma K ch^a sh^b with a = m+n,
 // b = m-n, sigma = (-1)^b; with FULL also d' and d'' (Appendix A.4 applied to
@@ -231,100 +132,7 @@ __device__ __forceinline__ void group_seed(unsigned pc, unsigned ps, unsigned z,
   }
 }
 
-// 2^e as a float for -126 <= e <= 127, 0 below (values that small times a
-// state below 2^32 are far under FP32 resolution of any sum they enter).
-__device__ __forceinline__ float pow2f(int e) {
-  return e < -126 ? 0.f : __int_as_float((min(e, 127) + 127) << 23);
-}
-
-// Extended-range power x^k = mant 2^expo (mant in [0.5, 1), or 0 for x = 0,
-// k > 0) by binary powering with the exponent carried as an integer, so
-// that powers far below the FP32 range keep their leading bits.
-__device__ __forceinline__ void xpow(float x, int k, float &mant, int &expo) {
-  int ex;
-  float xm = frexpf(x, &ex);
-  float rm = 1.f;
-  int re = 0;
-  while (k) {
-    if (k & 1) {
-      int t;
-      rm = frexpf(rm * xm, &t);
-      re += ex + t;
-    }
-    k >>= 1;
-    if (k) {
-      int t;
-      xm = frexpf(xm * xm, &t);
-      ex = 2 * ex + t;
-    }
-  }
-  if (rm == 0.f) re = 0;
-  int t;
-  mant = frexpf(rm, &t);
-  expo = re + t;
-}
-
-// Seeds of the rescaled recurrence (32-bit plans above L_J = 64).  The
-// powers come as (mantissa, exponent) from the extended-range tables: pc,
-// ps address ch^aa and sh^ba, pe is the byte offset of the exponent rows.
-// The states D0, D1, D2 of half h are the true seeds divided by 2^E_h,
-// E_h = the exponent of K ch^a sh^b, so the state of d starts near 1 however
-// small the true seed is; D1 and D2 keep their ratio to D0.
-template <bool FULL>
-__device__ __forceinline__ void group_seed_rs(unsigned pc, unsigned ps, unsigned pe, unsigned z,
-                                              v2<float> K, int aa, int ba, v2<float> &D0,
-                                              v2<float> &D1, v2<float> &D2, int &E0, int &E1) {
-  auto ldm = [&](unsigned a, float &m, int &e) {
-    float ef;
-    lds1(a, m);
-    lds1(a + pe, ef);
-    e = (int)ef;
-  };
-  float c0, c1, s0, sm1;
-  int ec0, ec1, es0, esm1;
-  ldm(pc, c0, ec0); ldm(pc + z, c1, ec1);
-  ldm(ps, s0, es0); ldm(ps - z, sm1, esm1);
-  int kex, key;
-  const float kmx = frexpf(K.x, &kex), kmy = frexpf(K.y, &key);
-  const int R0 = ec0 + es0, R1 = ec1 + esm1;  // reference exponents of ch^a sh^b
-  E0 = kex + R0;
-  E1 = key + R1;
-  const float g0 = kmx, g1 = -kmy;            // sigma K of both halves, mantissas
-  D0 = vset<float>(g0 * c0 * s0, g1 * c1 * sm1);
-  if (FULL) {
-    float c2, c3, cm1, cm2, s1, s2, sm2, sm3;
-    int ec2, ec3, ecm1, ecm2, es1, es2, esm2, esm3;
-    ldm(pc + 2 * z, c2, ec2); ldm(pc + 3 * z, c3, ec3);
-    ldm(pc - z, cm1, ecm1); ldm(pc - 2 * z, cm2, ecm2);
-    ldm(ps + z, s1, es1); ldm(ps + 2 * z, s2, es2);
-    ldm(ps - 2 * z, sm2, esm2); ldm(ps - 3 * z, sm3, esm3);
-    // ch^i sh^j relative to 2^R
-    auto rel = [](float cm, int ce, float sm, int se, int R) { return cm * sm * pow2f(ce + se - R); };
-    const float fa = (float)aa, fb = (float)ba;
-    // half 0: a = aa, b = ba; half 1: a = aa + 1, b = ba - 1
-    const float t1a = fb * rel(c1, ec1, sm1, esm1, R0), t2a = fa * rel(cm1, ecm1, s1, es1, R0);
-    const float t1b = (fb - 1.f) * rel(c2, ec2, sm2, esm2, R1), t2b = (fa + 1.f) * rel(c0, ec0, s0, es0, R1);
-    D1 = vset<float>(0.5f * g0 * (t1a - t2a), 0.5f * g1 * (t1b - t2b));
-    const float A0 = fa, B0 = fb, A1 = fa + 1.f, B1 = fb - 1.f;
-    const float u1a = B0 * (B0 - 1.f) * rel(c2, ec2, sm2, esm2, R0);
-    const float u2a = (B0 * (A0 + 1.f) + A0 * (B0 + 1.f)) * rel(c0, ec0, s0, es0, R0);
-    const float u3a = A0 * (A0 - 1.f) * rel(cm2, ecm2, s2, es2, R0);
-    const float u1b = B1 * (B1 - 1.f) * rel(c3, ec3, sm3, esm3, R1);
-    const float u2b = (B1 * (A1 + 1.f) + A1 * (B1 + 1.f)) * rel(c1, ec1, sm1, esm1, R1);
-    const float u3b = A1 * (A1 - 1.f) * rel(cm1, ecm1, s1, es1, R1);
-    D2 = vset<float>(0.25f * g0 * (u1a + u3a - u2a), 0.25f * g1 * (u1b + u3b - u2b));
-  }
-}
-
-// One staged degree entry of a partner group: c of both halves, the
-// recurrence coefficients (a, -b, -e) of the step to the next degree, and
-// -l(l+1) of the entry's own degree l.
-template <typename T> struct Coef {
-  v2<T> CR, CI, DR, DI;
-};
-template <typename T> struct Rec {
-  v2<T> A, NB, NE, NL;
-};
+// Entries interleaved: 8 c reals, then 8 recurrence reals.
 template <typename T> __device__ __forceinline__ void load_coef(unsigned a, Coef<T> &e) {
   lds4(a, e.CR, e.CI);
   lds4(a + 4 * sizeof(T), e.DR, e.DI);
@@ -333,40 +141,6 @@ template <typename T> __device__ __forceinline__ void load_rec(unsigned a, Rec<T
   lds4(a + 8 * sizeof(T), r.A, r.NB);
   lds4(a + 12 * sizeof(T), r.NE, r.NL);
 }
-// Z += c d (and c d', c d'' when FULL) for one entry; with ODE the third
-// sums take -l(l+1) c d (passed as D2 = -l(l+1) d) instead of c d''.
-template <typename T, bool FULL>
-__device__ __forceinline__ void accumulate(const Coef<T> &e, const v2<T> &D0, const v2<T> &D1,
-                                           const v2<T> &D2, v2<T> (&Z)[12]) {
-  Z[0] = vfma(e.CR, D0, Z[0]); Z[1] = vfma(e.CI, D0, Z[1]);
-  Z[2] = vfma(e.DR, D0, Z[2]); Z[3] = vfma(e.DI, D0, Z[3]);
-  if (FULL) {
-    Z[4] = vfma(e.CR, D1, Z[4]); Z[5] = vfma(e.CI, D1, Z[5]);
-    Z[6] = vfma(e.DR, D1, Z[6]); Z[7] = vfma(e.DI, D1, Z[7]);
-    Z[8] = vfma(e.CR, D2, Z[8]); Z[9] = vfma(e.CI, D2, Z[9]);
-    Z[10] = vfma(e.DR, D2, Z[10]); Z[11] = vfma(e.DI, D2, Z[11]);
-  }
-}
-// One recurrence step from (d^l, d^{l-1}) = (D, P); d^{l+1} overwrites P:
-//   d^{l+1} = t d - e p,  t = a x - b,
-//   d'^{l+1} = t d' - a s d - e p',  d''^{l+1} = t d'' - 2 a s d' - a x d - e p''.
-template <typename T, bool FULL, bool ODE = false>
-__device__ __forceinline__ void step_into(const Rec<T> &r, v2<T> X, v2<T> NS, v2<T> NX,
-                                          const v2<T> &D0, const v2<T> &D1, const v2<T> &D2,
-                                          v2<T> &P0, v2<T> &P1, v2<T> &P2) {
-  const v2<T> t = vfma(r.A, X, r.NB);
-  P0 = vfma(t, D0, vmul(r.NE, P0));
-  if (FULL && ODE) {
-    const v2<T> nAs = vmul(r.A, NS);
-    P1 = vfma(t, D1, vfma(nAs, D0, vmul(r.NE, P1)));
-  } else if (FULL) {
-    const v2<T> nAs = vmul(r.A, NS);
-    P1 = vfma(t, D1, vfma(nAs, D0, vmul(r.NE, P1)));
-    const v2<T> nAx = vmul(r.A, NX);
-    P2 = vfma(t, D2, vfma(vadd(nAs, nAs), D1, vfma(nAx, D0, vmul(r.NE, P2))));
-  }
-}
-
 // Sums over l = m..m+last of one partner group for one candidate: Z[0..3] =
 // sum d (Re c_mn, Im c_mn, Re c_nm, Im c_nm), then the same with d' (Z[4..7])
 // and d'' (Z[8..11]) when FULL; each a pair over the two halves.  With ODE
@@ -800,114 +574,6 @@ __device__ __forceinline__ void evaluate(const NewtonArgs &A, int L, const T *__
   __syncthreads();
 }
 
-// x mod 2 pi in [0, 2 pi).  The refinement only meets |x| < 4 pi (a wrapped
-// angle plus a clamped step, or plus pi after a reflection of beta), where a
-// few compare-and-add steps give the same result as x - 2 pi floor(x / 2 pi)
-// without a double-precision division; other inputs take that formula first.
-__device__ __forceinline__ double mod2pi_d(double x) {
-  const double t = 2.0 * M_PI;
-  if (!(x < 4.0 * t && x >= -4.0 * t)) x -= t * floor(x / t);
-  for (int k = 0; k < 4 && x >= t; ++k) x -= t;
-  for (int k = 0; k < 4 && x < 0.0; ++k) x += t;
-  return x;
-}
-
-__device__ __forceinline__ void wrap_d(double *v) {
-  double a = v[0], b = v[1], g = v[2];
-  if (b < 0) { b = -b; a += M_PI; g += M_PI; }
-  else if (b > M_PI) { b = 2.0 * M_PI - b; a += M_PI; g += M_PI; }
-  v[0] = mod2pi_d(a); v[1] = b; v[2] = mod2pi_d(g);
-}
-
-// Newton direction from grad g and Hessian H (row-major 3x3) in the solve
-// precision S; returns flag bits.  A Cholesky pivot of -H counts as positive
-// above piv_rel ||H||_F, set by the precision H was summed in (1e-12 for FP64
-// sums, 1e-6 for FP32 sums: above the rounding level of H's entries).
-template <typename S>
-__device__ __forceinline__ int newton_dir(const S *g, const S *H, int L, S *d, double piv_rel,
-                                          bool grad) {
-  S hn = 0;
-#pragma unroll
-  for (int i = 0; i < 9; ++i) hn += H[i] * H[i];
-  hn = sqrt(hn);
-  const S tol = S(piv_rel) * hn;
-  // Cholesky of A = -H
-  S a00 = -H[0], a10 = -H[3], a20 = -H[6], a11 = -H[4], a21 = -H[7], a22 = -H[8];
-  bool ok = !grad && a00 > tol;  // grad: the gradient method, never the Newton step
-  S L00 = 0, L10 = 0, L20 = 0, L11 = 0, L21 = 0, L22 = 0;
-  if (ok) {
-    L00 = sqrt(a00); L10 = a10 / L00; L20 = a20 / L00;
-    S p11 = a11 - L10 * L10;
-    ok = p11 > tol;
-    if (ok) {
-      L11 = sqrt(p11); L21 = (a21 - L20 * L10) / L11;
-      S p22 = a22 - L20 * L20 - L21 * L21;
-      ok = p22 > tol;
-      if (ok) L22 = sqrt(p22);
-    }
-  }
-  int fl = 0;
-  if (ok) {
-    S y0 = g[0] / L00;
-    S y1 = (g[1] - L10 * y0) / L11;
-    S y2 = (g[2] - L20 * y0 - L21 * y1) / L22;
-    S x2 = y2 / L22;
-    S x1 = (y1 - L21 * x2) / L11;
-    S x0 = (y0 - L10 * x1 - L20 * x2) / L00;
-    d[0] = x0; d[1] = x1; d[2] = x2;
-  } else {
-    fl = grad ? 0 : 2;
-#pragma unroll
-    for (int i = 0; i < 3; ++i) d[i] = hn > 0 ? g[i] / hn : S(0);
-  }
-  S nrm = sqrt(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]);
-  S cap = S(M_PI / (2.0 * (L + 1.0)));
-  if (nrm > cap) {
-    S f = cap / nrm;
-#pragma unroll
-    for (int i = 0; i < 3; ++i) d[i] *= f;
-  }
-  return fl;
-}
-
-// Candidate tid has C, grad, H of its current point in res: record C, stop on
-// a non-finite value (flag bit 0), take the Newton direction (solved in
-// precision S), stop the level when the increment is below step_tol, else
-// prepare the first trial (angles in FP64).
-template <typename S>
-__device__ __forceinline__ void start_step(int tid, int L, const NewtonArgs &A, SmemLayout &sm,
-                                           double piv_rel) {
-  const double *r = sm.res + 10 * tid;
-  const double C = r[0];
-  const S g[3] = {S(r[1]), S(r[2]), S(r[3])};
-  const S H[9] = {S(r[4]), S(r[5]), S(r[6]), S(r[5]), S(r[7]), S(r[8]), S(r[6]), S(r[8]), S(r[9])};
-  bool fin = true;
-#pragma unroll
-  for (int i = 0; i < 10; ++i) fin = fin && isfinite(r[i]);
-  sm.Cc[tid] = C;
-  if (!fin) {
-    sm.fl[tid] |= 1;
-    sm.state[tid] = ST_DEAD;
-    return;
-  }
-  S d[3];
-  sm.fl[tid] |= newton_dir<S>(g, H, L, d, piv_rel, A.grad != 0);
-  if (sqrt(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]) < S(A.tol)) {
-    sm.state[tid] = ST_STOP;
-    return;
-  }
-  double tr[3] = {sm.th[3 * tid] + (double)d[0], sm.th[3 * tid + 1] + (double)d[1],
-                  sm.th[3 * tid + 2] + (double)d[2]};
-  wrap_d(tr);
-#pragma unroll
-  for (int i = 0; i < 3; ++i) {
-    sm.del[3 * tid + i] = (double)d[i];
-    sm.tr[3 * tid + i] = tr[i];
-  }
-  sm.tries[tid] = 0;
-  sm.state[tid] = ST_TRIAL;
-}
-
 // Carves the refinement kernels' shared memory (layout of newton_smem_bytes).
 template <typename T, bool RS>
 __device__ __forceinline__ int *carve_smem(unsigned char *smem_raw, int P, int LJ, SmemLayout &sm) {
@@ -1001,8 +667,8 @@ __device__ __forceinline__ void newton_particle(const T *__restrict__ c, const T
     // the 3x3 solves of the final level run in FP64 in every plan
     const bool last = lev == A.nlev - 1;
     auto step_from = [&]() {
-      if (last) start_step<double>(tid, L, A, sm, piv_rel);
-      else start_step<T>(tid, L, A, sm, piv_rel);
+      if (last) start_step<double>(tid, L, A.tol, A.grad != 0, sm, piv_rel);
+      else start_step<T>(tid, L, A.tol, A.grad != 0, sm, piv_rel);
     };
     if (tid < P && need[tid]) {
       sm.steps[tid] = 0;
@@ -1138,11 +804,11 @@ static int newton_cpw(int P) { return P <= 16 ? 16 : 32; }
 // flushed below the FP32 range would otherwise grow into significant terms
 // (at L_J = 100 a seed under 2^-126 reaches 2.6e-4).
 constexpr int RESCALE_ABOVE_L = 64;
-static bool newton_rescaled(const Plan &p, size_t tsize) { return tsize == 4 && p.LJ > RESCALE_ABOVE_L; }
+bool newton_rescaled(const Plan &p) { return !p.fp64 && p.LJ > RESCALE_ABOVE_L; }
 
 static size_t newton_smem_bytes(const Plan &p, size_t tsize, int slots) {
   size_t P = p.P;
-  const size_t pw_rows = newton_rescaled(p, tsize) ? 4 : 2;
+  const size_t pw_rows = newton_rescaled(p) ? 4 : 2;
   size_t bytes = sizeof(double) * (3 * P * 3 + P + 10 * P);
   bytes += sizeof(int) * 5 * P;
   bytes = (bytes + 15) / 16 * 16;
@@ -1161,12 +827,16 @@ static int newton_slots(const Plan &p, size_t tsize) {
   return slots;
 }
 
-bool newton_fits(const Plan &p) { return newton_slots(p, p.fp64 ? 8 : 4) > 0; }
+int newton_slots(const Plan &p) { return newton_slots(p, p.fp64 ? 8 : 4); }
+size_t newton_smem(const Plan &p) { return newton_smem_bytes(p, p.fp64 ? 8 : 4, newton_slots(p)); }
+bool newton_fits(const Plan &p) { return newton_slots(p) > 0; }
 
 template <typename T>
 cudaError_t launch_newton(const Plan &p, const T *c, int B, const int *n_cand, double *euler,
                           double *score, int *cflags, long long *work, cudaStream_t st) {
   if (B == 0) return cudaSuccess;
+  cudaError_t e;
+  if (launch_newton_spread<T>(p, c, B, n_cand, euler, score, cflags, work, st, &e)) return e;
   NewtonArgs A;
   A.LJ = p.LJ; A.nlev = p.nlev; A.M = p.M; A.P = p.P;
   A.cpw = newton_cpw(p.P);
@@ -1179,7 +849,7 @@ cudaError_t launch_newton(const Plan &p, const T *c, int B, const int *n_cand, d
   A.nc = p.nc;
   size_t smem = newton_smem_bytes(p, sizeof(T), A.nslots);
   if constexpr (sizeof(T) == 4) {
-    if (newton_rescaled(p, sizeof(T))) {
+    if (newton_rescaled(p)) {
       cudaFuncSetAttribute(k_newton<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
       k_newton<T, true><<<B, NEWTON_THREADS, smem, st>>>(c, (const T *)p.rcoef, (const T *)p.seedK,
                                                          A, n_cand, euler, score, cflags, work);
@@ -1217,7 +887,7 @@ cudaError_t launch_newton_queue(const Plan &p, const T *c, int B, const int *n_c
                                              euler, score, cflags, work, order, B, ticket);
   };
   if constexpr (sizeof(T) == 4) {
-    if (newton_rescaled(p, sizeof(T))) { go(k_newton_queue<T, true>); return cudaGetLastError(); }
+    if (newton_rescaled(p)) { go(k_newton_queue<T, true>); return cudaGetLastError(); }
   }
   go(k_newton_queue<T, false>);
   return cudaGetLastError();
@@ -1233,6 +903,8 @@ template <typename T>
 cudaError_t launch_objective(const Plan &p, const T *c, int B, int L, int Q, const double *pts,
                              double *out, cudaStream_t st) {
   if (B == 0 || Q == 0) return cudaSuccess;
+  cudaError_t e;
+  if (launch_objective_spread<T>(p, c, B, L, Q, pts, out, st, &e)) return e;
   NewtonArgs A;
   A.LJ = p.LJ; A.nlev = p.nlev; A.M = p.M; A.P = p.P;
   A.cpw = newton_cpw(p.P);
@@ -1242,7 +914,7 @@ cudaError_t launch_objective(const Plan &p, const T *c, int B, int L, int Q, con
   A.tol = p.step_tol; A.acc_tol = p.accept_tol; A.grad = p.refine; A.nc = p.nc;
   size_t smem = newton_smem_bytes(p, sizeof(T), A.nslots);
   if constexpr (sizeof(T) == 4) {
-    if (newton_rescaled(p, sizeof(T))) {
+    if (newton_rescaled(p)) {
       cudaFuncSetAttribute(k_objective<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
       k_objective<T, true><<<B, NEWTON_THREADS, smem, st>>>(c, (const T *)p.rcoef,
                                                             (const T *)p.seedK, A, L, Q, pts, out);

@@ -206,6 +206,47 @@ __global__ void k_ptab_leg(int nt, int nlm, const int *leg, const T *in, T *out)
   out[t] = in[(long)j * nlm + l * (l + 1) / 2 + m];
 }
 
+// Constants of partner group g = (m, n_a), (m, n_b = n_a + 1) that the
+// refinement reads for every candidate, pairs over the two partners:
+//   0 sigma K, 2 sigma K / 2 (seed norms, sigma = (1, -1)), 4 m + n_a and
+//   m + n_a + 1, 6 m - n_a and m - n_a - 1 (the seeds' integer factors), 8 m n,
+//   10 (m - n)^2, 12 (m + n)^2, 14 m and 15 n_a (ints), then the image weights
+//   (W, -W u, -W v, -W u^2, -W u v, -W v^2) of (u, v) = (m, n) at 16 and of
+//   (n, m) at 28.  W is 2 (1 for m = n = 0), +-2 by the sign of the transposed
+//   function, 0 for an empty partner and for the image n = +-m already counted.
+template <typename T>
+__global__ void k_group_desc(int ngroups, const T *K, T *out) {
+  const int g = blockIdx.x * blockDim.x + threadIdx.x;
+  if (g >= ngroups) return;
+  const int m = tri_floor(g), na = 2 * (g - m * (m + 1) / 2) - m;
+  T *o = out + (long)GROUP_DESC * g;
+  for (int h = 0; h < 2; ++h) {
+    const int n = na + h;
+    const T sk = h ? -K[4 * g + 1] : K[4 * g];
+    o[h] = sk;
+    o[2 + h] = T(0.5) * sk;
+    o[4 + h] = T(m + na + h);
+    o[6 + h] = T(m - na - h);
+    o[8 + h] = T(m * n);
+    o[10 + h] = T((m - n) * (m - n));
+    o[12 + h] = T((m + n) * (m + n));
+    const int w1 = n > m ? 0 : m == 0 ? 1 : 2;
+    const int w2 = h ? (n < m ? -2 : 0) : (n == m || n == -m ? 0 : 2);
+    const int w[2] = {w1, w2}, u[2] = {m, n}, v[2] = {n, m};
+    for (int i = 0; i < 2; ++i) {
+      T *x = o + 16 + 12 * i + h;
+      x[0] = T(w[i]);
+      x[2] = T(-w[i] * u[i]);
+      x[4] = T(-w[i] * v[i]);
+      x[6] = T(-w[i] * u[i] * u[i]);
+      x[8] = T(-w[i] * u[i] * v[i]);
+      x[10] = T(-w[i] * v[i] * v[i]);
+    }
+  }
+  reinterpret_cast<int *>(o + 14)[0] = m;
+  reinterpret_cast<int *>(o + 15)[0] = na;
+}
+
 // out[e][k] = in[k][e] for ns x n tables.
 template <typename T>
 __global__ void k_transpose(int ns, long n, const T *in, T *out) {
@@ -256,6 +297,12 @@ cudaError_t build_tables(Plan &p, cudaStream_t st) {
     for (auto &c : cp)
       k_to_float<<<(unsigned)((c.n + 255) / 256), 256, 0, st>>>(c.src, (float *)c.dst, (long)c.n);
   }
+  if (p.fp64)
+    k_group_desc<double><<<(p.ngroups + 127) / 128, 128, 0, st>>>(p.ngroups, (const double *)p.seedK,
+                                                                   (double *)p.gdesc);
+  else
+    k_group_desc<float><<<(p.ngroups + 127) / 128, 128, 0, st>>>(p.ngroups, (const float *)p.seedK,
+                                                                  (float *)p.gdesc);
   {
     const unsigned nb = (unsigned)((n_softd + 255) / 256);
     if (p.fp64)
