@@ -9,7 +9,7 @@
 //      (mixed radix 4/2/3/5 Stockham passes along x, y and z, each line held
 //      in shared memory, loads and stores coalesced along x);
 //   2. X(k) = F(k) conj(U(k)) from Z(k) and Z(-k) (the two spectra of a
-//      packed pair), in place, one thread per conjugate pair;
+//      packed pair), in place, by the CTA that made both in its z transform;
 //   3. CC(t) = N^-3 Re sum_k X(k) e^{2 pi i k.t/N} (k in [-N/2, N/2)^3, the
 //      trigonometric interpolant of CC) only where it is needed, by three
 //      separable partial inverse DFTs (z, then y, then x): first on the
@@ -22,6 +22,7 @@
 // A pose kernel makes the rotated template u(x) = h(R^T (x - c0) + c0) and
 // the shifted template (S_tau h)(x) = h(x - tau) by trilinear interpolation.
 #include <math.h>
+#include <type_traits>
 #include "internal.cuh"
 
 namespace matcha {
@@ -48,23 +49,31 @@ __device__ __forceinline__ float add_rn(float a, float b) { return __fadd_rn(a, 
 // ---- volume pose ------------------------------------------------------------
 // out_b(x) = vol_b(R_b^T (x - c0) + c0 - s_b), trilinear, zero outside, one
 // thread per output voxel.  R (row-major [B][9]) and s ([B][3]) are nullable
-// (identity, zero).
+// (identity, zero).  Bound by the corner loads: a CTA takes a brick of 16 x 4 x 4
+// voxels, whose rotated corners share cache lines in all directions (a run of 256
+// along x does not), and all index arithmetic is 32-bit: corner indices are
+// clamped next to the box before the conversion (they are outside all the same),
+// the weights keep the unclamped coordinates.  The pose is converted once per CTA
+// (conversions from FP64 run at its rate).  96 volumes of 64^3 in FP32: rotated 652
+// -> 260 us, shifted 266 -> 240, of which the traffic is 30; the issue slots are 75%
+// busy (coordinates, eight guarded corners, weights).
+constexpr int POSE_X = 16, POSE_Y = 4, POSE_Z = 4;
 template <typename T>
-__global__ void __launch_bounds__(256)
-k_pose_volume(int N, const float *__restrict__ vol, long vstride, const double *__restrict__ R,
-              const double *__restrict__ sh, float *__restrict__ out) {
+__global__ void __launch_bounds__(POSE_X * POSE_Y * POSE_Z)
+k_pose_volume(int N, int nbx, int nby, const float *__restrict__ vol, long vstride,
+              const double *__restrict__ R, const double *__restrict__ sh, float *__restrict__ out) {
   const long b = blockIdx.y;
-  const long N2 = (long)N * N, N3 = N2 * N;
-  const long v = blockIdx.x * (long)blockDim.x + threadIdx.x;
-  if (v >= N3) return;
-  const int i = (int)(v % N), j = (int)((v / N) % N), k = (int)(v / N2);
+  const int bz = blockIdx.x / (nbx * nby), br = blockIdx.x - bz * nbx * nby, by = br / nbx;
+  const int i = (br - by * nbx) * POSE_X + threadIdx.x % POSE_X;
+  const int j = by * POSE_Y + threadIdx.x / POSE_X % POSE_Y;
+  const int k = bz * POSE_Z + threadIdx.x / (POSE_X * POSE_Y);
+  __shared__ T r[12];  // R, then s: converted once, conversions from FP64 run at its rate
+  if (threadIdx.x < 9) r[threadIdx.x] = R ? (T)R[9 * b + threadIdx.x] : T(threadIdx.x % 4 == 0);
+  else if (threadIdx.x < 12) r[threadIdx.x] = sh ? (T)sh[3 * b + threadIdx.x - 9] : T(0);
+  __syncthreads();
+  if (i >= N || j >= N || k >= N) return;
   const float *src = vol + b * vstride;
-  T r[9] = {1, 0, 0, 0, 1, 0, 0, 0, 1};
-  if (R)
-#pragma unroll
-    for (int q = 0; q < 9; ++q) r[q] = (T)R[9 * b + q];
-  T s0 = 0, s1 = 0, s2 = 0;
-  if (sh) { s0 = (T)sh[3 * b]; s1 = (T)sh[3 * b + 1]; s2 = (T)sh[3 * b + 2]; }
+  const T s0 = r[9], s1 = r[10], s2 = r[11];
   const T c0 = T(0.5) * (T)N;
   const T x = (T)i - c0, y = (T)j - c0, z = (T)k - c0;
   // column c of R dotted with (x, y, z), then + c0 - s, left to right
@@ -72,33 +81,38 @@ k_pose_volume(int N, const float *__restrict__ vol, long vstride, const double *
   T py = add_rn(add_rn(add_rn(add_rn(mul_rn(r[1], x), mul_rn(r[4], y)), mul_rn(r[7], z)), c0), -s1);
   T pz = add_rn(add_rn(add_rn(add_rn(mul_rn(r[2], x), mul_rn(r[5], y)), mul_rn(r[8], z)), c0), -s2);
   const T fx0 = floor(px), fy0 = floor(py), fz0 = floor(pz);
-  const long i0 = (long)fx0, j0 = (long)fy0, k0 = (long)fz0;
+  // -2 .. N + 1 (a NaN gives -2): past the box on either side with both corners
+  const T lo = T(-2), hi = (T)(N + 1);
+  const int i0 = (int)fmin(fmax(fx0, lo), hi), j0 = (int)fmin(fmax(fy0, lo), hi),
+            k0 = (int)fmin(fmax(fz0, lo), hi);
   const T tx = add_rn(px, -fx0), ty = add_rn(py, -fy0), tz = add_rn(pz, -fz0);
+  float val[8];
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    const int ii = i0 + (q & 1), jj = j0 + (q >> 1 & 1), kk = k0 + (q >> 2);
+    val[q] = 0.f;
+    if ((unsigned)ii < (unsigned)N && (unsigned)jj < (unsigned)N && (unsigned)kk < (unsigned)N)
+      val[q] = __ldg(src + (kk * N + jj) * N + ii);
+  }
   T acc = 0;
 #pragma unroll
-  for (int dz = 0; dz < 2; ++dz)
-#pragma unroll
-    for (int dy = 0; dy < 2; ++dy)
-#pragma unroll
-      for (int dx = 0; dx < 2; ++dx) {
-        const T w = mul_rn(mul_rn(dx ? tx : add_rn(T(1), -tx), dy ? ty : add_rn(T(1), -ty)),
-                           dz ? tz : add_rn(T(1), -tz));
-        const long ii = i0 + dx, jj = j0 + dy, kk = k0 + dz;
-        T val = 0;
-        if (ii >= 0 && jj >= 0 && kk >= 0 && ii < N && jj < N && kk < N)
-          val = (T)__ldg(src + (kk * N + jj) * N + ii);
-        acc = add_rn(acc, mul_rn(w, val));
-      }
-  out[b * N3 + v] = (float)acc;
+  for (int q = 0; q < 8; ++q) {
+    const int dx = q & 1, dy = q >> 1 & 1, dz = q >> 2;
+    const T w = mul_rn(mul_rn(dx ? tx : add_rn(T(1), -tx), dy ? ty : add_rn(T(1), -ty)),
+                       dz ? tz : add_rn(T(1), -tz));
+    acc = add_rn(acc, mul_rn(w, (T)val[q]));
+  }
+  out[b * (long)N * N * N + (k * N + j) * N + i] = (float)acc;
 }
 
 cudaError_t launch_pose_volumes(int N, const float *vol, int B, long vol_stride, const double *R,
                                 const double *shift, bool fp64, float *out, cudaStream_t st) {
   if (B <= 0) return cudaSuccess;
-  const long N3 = (long)N * N * N;
-  dim3 grid((unsigned)((N3 + 255) / 256), B);
-  if (fp64) k_pose_volume<double><<<grid, 256, 0, st>>>(N, vol, vol_stride, R, shift, out);
-  else k_pose_volume<float><<<grid, 256, 0, st>>>(N, vol, vol_stride, R, shift, out);
+  const int nbx = (N + POSE_X - 1) / POSE_X, nby = (N + POSE_Y - 1) / POSE_Y;
+  dim3 grid((unsigned)(nbx * nby * ((N + POSE_Z - 1) / POSE_Z)), B);
+  constexpr int threads = POSE_X * POSE_Y * POSE_Z;
+  if (fp64) k_pose_volume<double><<<grid, threads, 0, st>>>(N, nbx, nby, vol, vol_stride, R, shift, out);
+  else k_pose_volume<float><<<grid, threads, 0, st>>>(N, nbx, nby, vol, vol_stride, R, shift, out);
   return cudaGetLastError();
 }
 
@@ -108,95 +122,229 @@ struct FftDesc {
   int radix[16];
 };
 
-// Size-R DFT in place, V_q = sum_r v_r e^{sg 2 pi i q r / R} (sg = -1 forward).
-template <typename T>
-__device__ __forceinline__ void dft2(C2<T> *v, T) {
-  C2<T> a = v[0], b = v[1];
-  v[0] = cadd(a, b); v[1] = csub(a, b);
+// v, rounded: what follows may not be contracted with the operations that made it.
+__device__ __forceinline__ C2<float> rounded(C2<float> v) {
+  asm("" : "+f"(v.x), "+f"(v.y));
+  return v;
 }
-template <typename T>
-__device__ __forceinline__ void dft4(C2<T> *v, T sg) {
-  C2<T> s02 = cadd(v[0], v[2]), d02 = csub(v[0], v[2]);
-  C2<T> s13 = cadd(v[1], v[3]), d13 = cmuli(csub(v[1], v[3]), sg);
-  v[0] = cadd(s02, s13); v[2] = csub(s02, s13);
-  v[1] = cadd(d02, d13); v[3] = csub(d02, d13);
-}
-template <typename T>
-__device__ __forceinline__ void dft3(C2<T> *v, T sg) {
-  const T h3 = T(0.86602540378443864676);  // sin(2 pi / 3)
-  C2<T> t1 = cadd(v[1], v[2]), t2 = cmuli(csub(v[1], v[2]), sg * h3);
-  C2<T> a = csub(v[0], cscale(t1, T(0.5)));
-  v[0] = cadd(v[0], t1);
-  v[1] = cadd(a, t2);
-  v[2] = csub(a, t2);
-}
-template <typename T>
-__device__ __forceinline__ void dft5(C2<T> *v, T sg) {
-  const T c1 = T(0.30901699437494742410), c2 = T(-0.80901699437494742410);  // cos(2pi/5), cos(4pi/5)
-  const T s1 = T(0.95105651629515357212), s2 = T(0.58778525229247312917);   // sin(2pi/5), sin(4pi/5)
-  C2<T> t1 = cadd(v[1], v[4]), t2 = cadd(v[2], v[3]);
-  C2<T> t3 = csub(v[1], v[4]), t4 = csub(v[2], v[3]);
-  C2<T> a1 = cadd(v[0], cadd(cscale(t1, c1), cscale(t2, c2)));
-  C2<T> a2 = cadd(v[0], cadd(cscale(t1, c2), cscale(t2, c1)));
-  C2<T> b1 = cmuli(cadd(cscale(t3, s1), cscale(t4, s2)), sg);
-  C2<T> b2 = cmuli(csub(cscale(t3, s2), cscale(t4, s1)), sg);
-  v[0] = cadd(v[0], cadd(t1, t2));
-  v[1] = cadd(a1, b1); v[4] = csub(a1, b1);
-  v[2] = cadd(a2, b2); v[3] = csub(a2, b2);
+__device__ __forceinline__ C2<double> rounded(C2<double> v) {
+  asm("" : "+d"(v.x), "+d"(v.y));
+  return v;
 }
 
-// One Stockham autosort pass of radix R over NB lines (line stride LS) of
-// length N: butterfly j of a line reads A[j + r N/R], applies the twiddles
-// e^{sg 2 pi i k r / (Ns R)} (k = j mod Ns, Ns = product of earlier radices)
-// and writes B[(j / Ns) Ns R + k + r Ns].
+// Size-R DFT in place, V_q = sum_r v_r e^{-2 pi i q r / R}.
 template <int R, typename T>
-__device__ __forceinline__ void fft_pass(const C2<T> *A, C2<T> *Bv, int N, int LS, int NB, int Ns,
-                                         const C2<T> *__restrict__ tw, T sg) {
-  const int NR = N / R, span = N / (Ns * R);
-  for (int t = threadIdx.x; t < NB * NR; t += blockDim.x) {
-    const int line = t / NR, j = t - line * NR;
-    const int k = j % Ns;
-    const C2<T> *a = A + line * LS;
-    C2<T> v[R];
-#pragma unroll
-    for (int r = 0; r < R; ++r) v[r] = a[j + r * NR];
-    if (Ns > 1) {
-#pragma unroll
-      for (int r = 1; r < R; ++r) {
-        C2<T> w = tw[k * r * span];  // e^{-2 pi i k r / (Ns R)}
-        if (sg > 0) w.y = -w.y;
-        v[r] = cmul(v[r], w);
-      }
-    }
-    if (R == 2) dft2(v, sg);
-    else if (R == 3) dft3(v, sg);
-    else if (R == 4) dft4(v, sg);
-    else dft5(v, sg);
-    C2<T> *o = Bv + line * LS + (j / Ns) * Ns * R + k;
-#pragma unroll
-    for (int r = 0; r < R; ++r) o[r * Ns] = v[r];
+__device__ __forceinline__ void dft(C2<T> *v) {
+  if (R == 2) {
+    C2<T> a = v[0], b = v[1];
+    v[0] = cadd(a, b); v[1] = csub(a, b);
+  } else if (R == 4) {
+    C2<T> s02 = cadd(v[0], v[2]), d02 = csub(v[0], v[2]);
+    C2<T> s13 = cadd(v[1], v[3]), d13 = cmuli(csub(v[1], v[3]), T(-1));
+    v[0] = cadd(s02, s13); v[2] = csub(s02, s13);
+    v[1] = cadd(d02, d13); v[3] = csub(d02, d13);
+  } else if (R == 3) {
+    const T h3 = T(0.86602540378443864676);  // sin(2 pi / 3)
+    C2<T> t1 = cadd(v[1], v[2]), t2 = cmuli(csub(v[1], v[2]), -h3);
+    C2<T> a = csub(v[0], cscale(t1, T(0.5)));
+    v[0] = cadd(v[0], t1);
+    v[1] = cadd(a, t2);
+    v[2] = csub(a, t2);
+  } else {
+    const T c1 = T(0.30901699437494742410), c2 = T(-0.80901699437494742410);  // cos(2pi/5), cos(4pi/5)
+    const T s1 = T(0.95105651629515357212), s2 = T(0.58778525229247312917);   // sin(2pi/5), sin(4pi/5)
+    C2<T> t1 = cadd(v[1], v[4]), t2 = cadd(v[2], v[3]);
+    C2<T> t3 = csub(v[1], v[4]), t4 = csub(v[2], v[3]);
+    C2<T> a1 = cadd(v[0], cadd(cscale(t1, c1), cscale(t2, c2)));
+    C2<T> a2 = cadd(v[0], cadd(cscale(t1, c2), cscale(t2, c1)));
+    C2<T> b1 = rounded(cmuli(cadd(cscale(t3, s1), cscale(t4, s2)), T(-1)));
+    C2<T> b2 = rounded(cmuli(csub(cscale(t3, s2), cscale(t4, s1)), T(-1)));
+    v[0] = cadd(v[0], cadd(t1, t2));
+    v[1] = cadd(a1, b1); v[4] = csub(a1, b1);
+    v[2] = cadd(a2, b2); v[3] = csub(a2, b2);
   }
 }
 
-// Length-N transforms of NB lines of each volume along `axis` (0 x, 1 y,
-// 2 z), in place.  Axis 0: NB consecutive rows; axes 1 and 2: NB
-// consecutive x columns of one z plane (axis 1) or one y plane (axis 2), so
-// every global access runs along x.  With fre/fim given (forward x pass
-// only) the input is the packed pair fre + i fim of float volumes.
+// v w rounded as written, whatever follows (left to the compiler the outer
+// operation could join the transform's additions, which would change last bits).
+__device__ __forceinline__ C2<float> twiddle(C2<float> v, C2<float> w) {
+  return {__fmaf_rn(v.x, w.x, -__fmul_rn(v.y, w.y)), __fmaf_rn(v.x, w.y, __fmul_rn(v.y, w.x))};
+}
+__device__ __forceinline__ C2<double> twiddle(C2<double> v, C2<double> w) {
+  return {__fma_rn(v.x, w.x, -__dmul_rn(v.y, w.y)), __fma_rn(v.x, w.y, __dmul_rn(v.y, w.x))};
+}
+
+// One Stockham autosort pass of radix R over NB lines of length N: butterfly j of
+// a line reads elements j + r N/R, applies the twiddles e^{-2 pi i k r / (Ns R)} (k =
+// j mod Ns, Ns = product of earlier radices) and writes elements (j / Ns) Ns R + k +
+// r Ns.  ld(line, e) and st(line, e, v): the elements.  Neighbouring threads take
+// neighbouring lines, and a thread stays on its line where the lines divide the
+// block.  tw: the twiddles in shared memory.
+template <typename F>
+__device__ __forceinline__ void fft_tasks(int n, int NB, F &&task) {
+  if (blockDim.x % NB == 0) {
+    const int j0 = threadIdx.x / NB, line = threadIdx.x - j0 * NB;
+    for (int j = j0; j < n; j += blockDim.x / NB) task(line, j);
+    return;
+  }
+  const FastDiv dl(NB);
+  for (int t = threadIdx.x; t < NB * n; t += blockDim.x) {
+    const int j = dl.div(t);
+    task(t - j * NB, j);
+  }
+}
+template <int R, typename T, typename Ld, typename St>
+__device__ __forceinline__ void fft_pass(Ld ld, St st, int N, int NB, int Ns, const C2<T> *tw) {
+  const FastDiv dn(Ns);
+  if constexpr (R != 16) {
+    const int NR = N / R, span = N / (Ns * R);
+    fft_tasks(NR, NB, [&](int line, int j) {
+      const int jn = dn.div(j), k = j - jn * Ns;
+      C2<T> v[R];
+#pragma unroll
+      for (int r = 0; r < R; ++r) v[r] = ld(line, j + r * NR);
+      if (Ns > 1)
+#pragma unroll
+        for (int r = 1; r < R; ++r) v[r] = twiddle(v[r], tw[k * r * span]);
+      dft<R>(v);
+#pragma unroll
+      for (int r = 0; r < R; ++r) st(line, jn * Ns * R + k + r * Ns, v[r]);
+    });
+  } else {
+    // two radix-4 passes in one, the 16 values between them in registers: the first
+    // one's butterflies j + q N/16 write what the second one's, k + r Ns, read
+    const int M = N / 16, s1 = N / (Ns * 4), s2 = N / (Ns * 16);
+    fft_tasks(M, NB, [&](int line, int j) {
+      const int jn = dn.div(j), k = j - jn * Ns;
+      C2<T> v[4][4];  // [q][r]
+#pragma unroll
+      for (int r = 0; r < 4; ++r)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) v[q][r] = ld(line, j + (4 * r + q) * M);
+      if (Ns > 1)
+#pragma unroll
+        for (int r = 1; r < 4; ++r) {
+          const C2<T> w = tw[k * r * s1];
+#pragma unroll
+          for (int q = 0; q < 4; ++q) v[q][r] = twiddle(v[q][r], w);
+        }
+#pragma unroll
+      for (int q = 0; q < 4; ++q) dft<4>(v[q]);
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        C2<T> u[4] = {v[0][r], v[1][r], v[2][r], v[3][r]};
+#pragma unroll
+        for (int q = 1; q < 4; ++q) u[q] = twiddle(u[q], tw[(k + r * Ns) * q * s2]);
+        dft<4>(u);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) st(line, jn * Ns * 16 + k + (r + 4 * q) * Ns, u[q]);
+      }
+    });
+  }
+}
+
+// All passes of NB lines in the buffers src and dst (shared memory; element e of
+// line l at l * ls + e * es, ls odd or es a row of lines, so that no banks collide).
+// The first pass reads src, or gld(line, e) if one is given; the last leaves the
+// result in src, or hands it to gst(line, e, v) and needs no more of the block.
+struct InSmem {};
+template <typename T, typename Gld = InSmem, typename Gst = InSmem>
+__device__ __forceinline__ void fft_lines(C2<T> *&src, C2<T> *&dst, const FftDesc &fd, int ls, int es,
+                                          int NB, const C2<T> *tw, Gld gld = {}, Gst gst = {}) {
+  const int N = fd.N;
+  int Ns = 1;
+  for (int q = 0; q < fd.npass; ++q) {
+    int R = fd.radix[q];
+    const bool head = q == 0;
+    if (R == 4 && q + 1 < fd.npass && fd.radix[q + 1] == 4) {
+      R = 16;
+      ++q;
+    }
+    const bool tail = q + 1 >= fd.npass;
+    auto sld = [=](int l, int e) { return src[l * ls + e * es]; };
+    auto sst = [=](int l, int e, C2<T> v) { dst[l * ls + e * es] = v; };
+    auto pass = [&](auto ld, auto st) {
+      if (R == 16) fft_pass<16>(ld, st, N, NB, Ns, tw);
+      else if (R == 4) fft_pass<4>(ld, st, N, NB, Ns, tw);
+      else if (R == 2) fft_pass<2>(ld, st, N, NB, Ns, tw);
+      else if (R == 3) fft_pass<3>(ld, st, N, NB, Ns, tw);
+      else fft_pass<5>(ld, st, N, NB, Ns, tw);
+    };
+    constexpr bool GL = !std::is_same<Gld, InSmem>::value, GS = !std::is_same<Gst, InSmem>::value;
+    static_assert(!(GL && GS), "one of the two");
+    if constexpr (GL) {
+      if (head) pass(gld, sst);
+      else pass(sld, sst);
+    } else if constexpr (GS) {
+      if (tail) {
+        pass(sld, gst);
+        return;
+      }
+      pass(sld, sst);
+    } else {
+      pass(sld, sst);
+    }
+    __syncthreads();
+    C2<T> *tmp = src; src = dst; dst = tmp;
+    Ns *= R;
+  }
+}
+
+// Forward x and y transforms of one z plane of the packed pair fre + i fim: the
+// plane stays in shared memory between them, so the volume crosses HBM once.  A
+// thread has 16 voxels of each volume in flight (loads of a loop that did not batch
+// them left the warps waiting: 208 us), and the last y pass stores to memory.  96
+// pairs of 64^3 in FP32: two passes of k_fft_axis 532 us, this 141, of which the
+// traffic is 60; then the issue of the butterflies (72% busy).
+template <typename T>
+__global__ void __launch_bounds__(256)
+k_fft_plane(C2<T> *__restrict__ data, const float *__restrict__ fre, const float *__restrict__ fim,
+            const __grid_constant__ FftDesc fd, const C2<T> *__restrict__ twg) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int N = fd.N, LS = N | 1, N2 = N * N;
+  C2<T> *src = reinterpret_cast<C2<T> *>(smem_raw), *dst = src + N * LS, *tw = dst + N * LS;
+  const long o = blockIdx.y * (long)N2 * N + blockIdx.x * (long)N2;
+  const FastDiv dN(N);
+  constexpr int U = 16;  // voxels of a thread in flight
+  for (int t0 = threadIdx.x; t0 < N2; t0 += U * blockDim.x) {
+    float re[U], im[U];
+#pragma unroll
+    for (int q = 0; q < U; ++q) {
+      const int t = t0 + q * blockDim.x;
+      re[q] = t < N2 ? __ldg(fre + o + t) : 0.f;
+      im[q] = t < N2 ? __ldg(fim + o + t) : 0.f;
+    }
+#pragma unroll
+    for (int q = 0; q < U; ++q) {
+      const int t = t0 + q * blockDim.x;
+      if (t < N2) src[t + dN.div(t) * (LS - N)] = C2<T>{(T)re[q], (T)im[q]};
+    }
+  }
+  for (int t = threadIdx.x; t < N; t += blockDim.x) tw[t] = twg[t];
+  __syncthreads();
+  fft_lines(src, dst, fd, LS, 1, N, tw);
+  C2<T> *out = data + o;
+  fft_lines(src, dst, fd, 1, LS, N, tw, InSmem{}, [=](int l, int e, C2<T> v) { out[e * N + l] = v; });
+}
+
+// Length-N transforms of NB lines of each volume along `axis` (0 x, 1 y), in
+// place, for planes that do not fit in shared memory.  Axis 0: NB consecutive
+// rows of the packed pair fre + i fim of float volumes; axis 1: NB consecutive x
+// columns of one z plane, so every global access runs along x.
 template <typename T>
 __global__ void __launch_bounds__(256)
 k_fft_axis(C2<T> *__restrict__ data, const float *__restrict__ fre, const float *__restrict__ fim,
-           int axis, FftDesc fd, const C2<T> *__restrict__ tw, int NB, T sg) {
+           int axis, const __grid_constant__ FftDesc fd, const C2<T> *__restrict__ twg, int NB) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int N = fd.N, LS = N + 1;
-  C2<T> *bufA = reinterpret_cast<C2<T> *>(smem_raw);
-  C2<T> *bufB = bufA + NB * LS;
+  const int N = fd.N, LS = N | 1;
+  C2<T> *src = reinterpret_cast<C2<T> *>(smem_raw), *dst = src + NB * LS, *tw = dst + NB * LS;
+  for (int t = threadIdx.x; t < N; t += blockDim.x) tw[t] = twg[t];
   const long b = blockIdx.y;
   const long N2 = (long)N * N, N3 = N2 * N;
   C2<T> *vol = data + b * N3;
   const int tid = threadIdx.x, NT = blockDim.x;
   const long g = blockIdx.x;
-  long row0 = 0, ob = 0, es = 1;
+  long row0 = 0, ob = 0;
   int x0 = 0;
   if (axis == 0) {
     row0 = g * NB;
@@ -204,83 +352,100 @@ k_fft_axis(C2<T> *__restrict__ data, const float *__restrict__ fre, const float 
     const int ntile = (N + NB - 1) / NB;
     const long outer = g / ntile;
     x0 = (int)(g - outer * ntile) * NB;
-    es = axis == 1 ? N : N2;
-    ob = axis == 1 ? outer * N2 : outer * N;
+    ob = outer * N2;
   }
-  // load
+  const FastDiv dN(axis == 0 ? N : NB);
+  auto at = [&](int idx, int &line, int &e, long &off) {
+    const int q = dN.div(idx), w = idx - q * dN.d;
+    line = axis == 0 ? q : w;
+    e = axis == 0 ? w : q;
+    off = axis == 0 ? (row0 + line) * N + e : ob + (long)e * N + x0 + line;
+    return axis == 0 ? row0 + line < N2 : x0 + line < N;
+  };
   for (int idx = tid; idx < NB * N; idx += NT) {
     int line, e;
     long off;
-    bool ok;
-    if (axis == 0) {
-      line = idx / N; e = idx - line * N;
-      ok = row0 + line < N2;
-      off = (row0 + line) * N + e;
-    } else {
-      e = idx / NB; line = idx - e * NB;
-      ok = x0 + line < N;
-      off = ob + e * es + x0 + line;
-    }
     C2<T> v{T(0), T(0)};
-    if (ok) {
-      if (fre) v = C2<T>{(T)__ldg(fre + b * N3 + off), (T)__ldg(fim + b * N3 + off)};
-      else v = vol[off];
-    }
-    bufA[line * LS + e] = v;
+    if (at(idx, line, e, off))
+      v = axis == 0 ? C2<T>{(T)__ldg(fre + b * N3 + off), (T)__ldg(fim + b * N3 + off)} : vol[off];
+    src[line * LS + e] = v;
   }
   __syncthreads();
-  C2<T> *src = bufA, *dst = bufB;
-  int Ns = 1;
-  for (int q = 0; q < fd.npass; ++q) {
-    const int R = fd.radix[q];
-    if (R == 4) fft_pass<4>(src, dst, N, LS, NB, Ns, tw, sg);
-    else if (R == 2) fft_pass<2>(src, dst, N, LS, NB, Ns, tw, sg);
-    else if (R == 3) fft_pass<3>(src, dst, N, LS, NB, Ns, tw, sg);
-    else fft_pass<5>(src, dst, N, LS, NB, Ns, tw, sg);
-    __syncthreads();
-    C2<T> *tmp = src; src = dst; dst = tmp;
-    Ns *= R;
-  }
-  // store
+  fft_lines(src, dst, fd, LS, 1, NB, tw);
   for (int idx = tid; idx < NB * N; idx += NT) {
     int line, e;
     long off;
-    bool ok;
-    if (axis == 0) {
-      line = idx / N; e = idx - line * N;
-      ok = row0 + line < N2;
-      off = (row0 + line) * N + e;
-    } else {
-      e = idx / NB; line = idx - e * NB;
-      ok = x0 + line < N;
-      off = ob + e * es + x0 + line;
-    }
-    if (ok) vol[off] = src[line * LS + e];
+    if (at(idx, line, e, off)) vol[off] = src[line * LS + e];
   }
 }
 
-// X(k) = F(k) conj(U(k)) in place from the packed spectrum Z = FFT(f + i u):
-// F = (Z(k) + conj Z(-k)) / 2, U = (Z(k) - conj Z(-k)) / (2i), so
-// X(k) = (i/4) (Z(k) + conj Z(-k)) (conj Z(k) - Z(-k)) and X(-k) = conj X(k)
-// (CC is real).  One thread per conjugate pair (the smaller linear index).
+// The z transform and, still in shared memory, the cross spectrum: X(k) = F(k)
+// conj(U(k)) from the packed spectrum Z = FFT(f + i u): F = (Z(k) + conj Z(-k)) / 2,
+// U = (Z(k) - conj Z(-k)) / (2i), so X(k) = (i/4) (Z(k) + conj Z(-k)) (conj Z(k) -
+// Z(-k)) and X(-k) = conj X(k) (CC is real).  A CTA takes NB columns kx of plane ky
+// and the columns -kx of plane -ky (the columns 0 .. N/2 where ky = -ky), so that
+// both members of every conjugate pair are at hand; the member with the smaller
+// linear index plays k.  96 volumes of 64^3 in FP32: 383 us as a transform and a
+// pass of its own, 112 here (traffic 60; 65% of the issue slots): the first pass reads
+// memory directly, with no staging copy and barrier before it.
 template <typename T>
-__global__ void __launch_bounds__(256) k_cross_spectrum(C2<T> *__restrict__ Z, int N) {
-  const long b = blockIdx.y;
-  const long N2 = (long)N * N, N3 = N2 * N;
-  const long q = blockIdx.x * (long)blockDim.x + threadIdx.x;
-  if (q >= N3) return;
-  const int kx = (int)(q % N), ky = (int)((q / N) % N), kz = (int)(q / N2);
-  const int mx = kx ? N - kx : 0, my = ky ? N - ky : 0, mz = kz ? N - kz : 0;
-  const long q2 = ((long)mz * N + my) * N + mx;
-  if (q2 < q) return;
-  C2<T> *zb = Z + b * N3;
-  const C2<T> A = zb[q], C = zb[q2];
-  const C2<T> s{A.x + C.x, A.y - C.y};    // Z(k) + conj Z(-k)
-  const C2<T> d{A.x - C.x, -A.y - C.y};   // conj Z(k) - Z(-k)
-  const C2<T> p = cmul(s, d);
-  const C2<T> X{-T(0.25) * p.y, T(0.25) * p.x};
-  zb[q] = X;
-  if (q2 != q) zb[q2] = C2<T>{X.x, -X.y};
+__global__ void __launch_bounds__(128)
+k_fft_cross(C2<T> *__restrict__ Z, const __grid_constant__ FftDesc fd, const C2<T> *__restrict__ twg,
+            int NB) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int N = fd.N, N2 = N * N, L2 = 2 * NB, tid = threadIdx.x;
+  C2<T> *src = reinterpret_cast<C2<T> *>(smem_raw), *dst = src + N * L2, *tw = dst + N * L2;
+  C2<T> *zb = Z + blockIdx.y * (long)N2 * N;
+  // planes 0 and (N even) N/2 are their own partners and come first
+  const int nself = N % 2 ? 1 : 2, tself = (N / 2 + NB) / NB, tfull = (N + NB - 1) / NB;
+  int ky, x0, nx;
+  if ((int)blockIdx.x < nself * tself) {
+    const int q = blockIdx.x / tself;
+    ky = q ? N / 2 : 0;
+    x0 = (blockIdx.x - q * tself) * NB;
+    nx = N / 2 + 1;
+  } else {
+    const int g = blockIdx.x - nself * tself, q = g / tfull;
+    ky = q + 1;
+    x0 = (g - q * tfull) * NB;
+    nx = N;
+  }
+  const int my = ky ? N - ky : 0;
+  for (int t = tid; t < N; t += blockDim.x) tw[t] = twg[t];
+  // this thread's line w (2 NB divides the block): column x0 + w of plane ky (w <
+  // NB), or the mirror of column x0 + w - NB in plane -ky
+  const int z0 = tid / L2, w = tid - z0 * L2, dz = blockDim.x / L2, x = x0 + (w < NB ? w : w - NB);
+  const int mx = x ? N - x : 0;
+  const bool live = x < nx;
+  C2<T> *col = zb + (w < NB ? ky * N + x : my * N + mx);
+  __syncthreads();
+  // the first pass reads the thread's line w from memory
+  fft_lines(src, dst, fd, 1, L2, L2, tw,
+            [=](int, int kz) { return live ? col[kz * N2] : C2<T>{T(0), T(0)}; });
+  const bool own = ky == my && x == mx;  // the column is its own partner
+  if (live) {
+    // the pairs (kz of the column, -kz of its partner) are shared between the
+    // threads of the two lines: first halves of kz here, second halves there
+    for (int q = w < NB ? z0 : z0 + dz; q < N; q += 2 * dz) {
+      const int kz = q, mz = kz ? N - kz : 0, wa = w < NB ? w : w - NB;
+      if (own && mz < kz) continue;
+      C2<T> *pa = src + kz * L2 + wa, *pc = src + mz * L2 + (own ? wa : NB + wa);
+      // the smaller linear index first
+      const bool first = kz != mz ? kz < mz : ky != my ? ky < my : x <= mx;
+      if (!first) { C2<T> *tmp = pa; pa = pc; pc = tmp; }
+      const C2<T> A = *pa, C = *pc;
+      const C2<T> s{A.x + C.x, A.y - C.y};    // Z(k) + conj Z(-k)
+      const C2<T> d{A.x - C.x, -A.y - C.y};   // conj Z(k) - Z(-k)
+      const C2<T> p = cmul(s, d);
+      const C2<T> X{-T(0.25) * p.y, T(0.25) * p.x};
+      *pa = X;
+      if (pa != pc) *pc = C2<T>{X.x, -X.y};
+    }
+  }
+  __syncthreads();
+  if (live && !(own && w >= NB))  // its own partner: stored once
+#pragma unroll 8
+    for (int kz = z0; kz < N; kz += dz) col[kz * N2] = src[kz * L2 + w];
 }
 
 // Grid point j of axis a of particle b: t = org[b][a] + (j + j0) / den (org
@@ -290,67 +455,126 @@ __device__ __forceinline__ double grid_t(const double *org, long b, int a, int j
 }
 
 // E[b][a][k][j] = e^{2 pi i kk t / N} at the grid points t, kk = k or k - N
-// (the symmetric frequency range); a = 0, 1, 2 for the x, y, z components.
+// (the symmetric frequency range); a = 0, 1, 2 for the x, y, z components.  One
+// run of CTAs per (b, a); the points' FP64 divisions are made once per CTA.
 template <typename T>
 __global__ void __launch_bounds__(256)
-k_idft_factors(C2<T> *__restrict__ E, int N, int nt, int B, const double *__restrict__ org,
-               int j0, int den) {
-  const long tot = (long)B * 3 * N * nt;
-  const long q = blockIdx.x * (long)blockDim.x + threadIdx.x;
-  if (q >= tot) return;
-  const int j = (int)(q % nt);
-  const int k = (int)((q / nt) % N);
-  const int a = (int)((q / ((long)nt * N)) % 3);
-  const long b = q / ((long)3 * N * nt);
-  const int kk = k < (N + 1) / 2 ? k : k - N;
-  const double t = grid_t(org, b, a, j, j0, den);
+k_idft_factors(C2<T> *__restrict__ E, int N, int nt, const double *__restrict__ org, int j0, int den) {
+  __shared__ double ts[256];
+  const int run = (N * nt + blockDim.x - 1) / blockDim.x;  // CTAs per (b, a)
+  const int ba = blockIdx.x / run, b = ba / 3, a = ba - 3 * b;
+  const bool pow2 = (N & (N - 1)) == 0;
+  const double inv = 1.0 / N;
+  for (int j = threadIdx.x; j < nt; j += blockDim.x) ts[j] = grid_t(org, b, a, j, j0, den);
+  __syncthreads();
+  const FastDiv dt(nt);
+  const int q = (blockIdx.x - ba * run) * blockDim.x + threadIdx.x;
+  if (q >= N * nt) return;
+  const int k = dt.div(q), kk = k < (N + 1) / 2 ? k : k - N;
+  const double u = 2.0 * kk * ts[q - k * nt];
+  const double x = pow2 ? u * inv : u / N;  // the same bits: 1/N is exact
   T s, c;
   if (sizeof(T) == 8) {
     double sd, cd;
-    sincospi(2.0 * kk * t / N, &sd, &cd);
+    sincospi(x, &sd, &cd);
     s = (T)sd; c = (T)cd;
   } else {
     float sf, cf;
-    sincospif((float)(2.0 * kk * t / N), &sf, &cf);
+    sincospif((float)x, &sf, &cf);
     s = (T)sf; c = (T)cf;
   }
-  E[q] = C2<T>{c, s};
+  E[(long)ba * N * nt + q] = C2<T>{c, s};
 }
 
+// v e added to a, each part's two products fused once and rounded before they are
+// added: a.x + (v.x e.x - v.y e.y), a.y + (v.y e.x + v.x e.y), the first product of
+// each exact in the fused sum; q holds (e.x, e.x, -e.y, e.y).
+__device__ __forceinline__ float2 cmac(float2 a, float2 v, const float4 &q) {
+  const float2 m = __fmul2_rn(make_float2(v.y, v.x), make_float2(q.z, q.w));
+  return __fadd2_rn(a, __ffma2_rn(v, make_float2(q.x, q.y), m));
+}
+struct alignas(16) Double4 { double x, y, z, w; };
+__device__ __forceinline__ double2 cmac(double2 a, double2 v, const Double4 &q) {
+  return make_double2(__dadd_rn(a.x, __fma_rn(v.x, q.x, __dmul_rn(v.y, q.z))),
+                      __dadd_rn(a.y, __fma_rn(v.y, q.y, __dmul_rn(v.x, q.w))));
+}
+template <typename T> struct CPair;
+template <> struct CPair<float> { typedef float2 type; typedef float4 quad; };
+template <> struct CPair<double> { typedef double2 type; typedef Double4 quad; };
+
 // out[b][a][j][c] = sum_k in[b][a][k][c] E[b][axis][k][j]: the partial inverse
-// DFT along a middle (y) or outer (z) axis.  One CTA per (a, tile of TC
-// columns, b); the tile's N x TC inputs and the N x nt factors sit in shared
-// memory.
-template <typename T>
-__global__ void __launch_bounds__(256)
+// DFT along a middle (y) or outer (z) axis.  A thread takes CB columns c, JB grid
+// points j at a time in registers against the factors in shared memory (one 16-byte
+// broadcast per CB products of three packed operations); four rows k of its columns
+// are in flight while the four before are multiplied.  es: elements between the
+// particles' factors (0: shared).  96 volumes of 64^3 in FP32, 11 and 29 grid points:
+// the z stage 139 and 171 us -> 76 and 97 (one column per thread 97 and 117; two
+// without the loads ahead 128 and 143), then bound by its FMAs (floor 33) and, past
+// 16 points, by reading the volume again.
+template <typename T, int JB, int CB>
+__global__ void __launch_bounds__(128)
 k_idft_mid(const C2<T> *__restrict__ in, C2<T> *__restrict__ out, const C2<T> *__restrict__ E,
-           int N, int nt, int A, long C, int TC, int axis) {
+           int N, int nt, int A, int C, int axis, long es) {
+  typedef typename CPair<T>::type P2;
+  typedef typename CPair<T>::quad Q;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  C2<T> *slab = reinterpret_cast<C2<T> *>(smem_raw);  // [N][TC]
-  C2<T> *Es = slab + (long)N * TC;                     // [N][nt]
-  const long b = blockIdx.y;
-  const long ntile = (C + TC - 1) / TC;
-  const long a = blockIdx.x / ntile, c0 = (blockIdx.x - a * ntile) * (long)TC;
-  const C2<T> *src = in + (b * A + a) * (long)N * C;
-  const C2<T> *eb = E + ((b * 3 + axis) * (long)N) * nt;
-  const int tid = threadIdx.x, NT = blockDim.x;
-  for (int idx = tid; idx < N * TC; idx += NT) {
-    const int k = idx / TC, c = idx - k * TC;
-    slab[idx] = c0 + c < C ? src[(long)k * C + c0 + c] : C2<T>{T(0), T(0)};
-  }
-  for (int idx = tid; idx < N * nt; idx += NT) Es[idx] = eb[idx];
-  __syncthreads();
-  C2<T> *dstb = out + (b * A + a) * (long)nt * C;
-  for (int o = tid; o < nt * TC; o += NT) {
-    const int j = o / TC, c = o - j * TC;
-    if (c0 + c >= C) continue;
-    T re = 0, im = 0;
-    for (int k = 0; k < N; ++k) {
-      const C2<T> v = slab[k * TC + c], e = Es[k * nt + j];
-      re += v.x * e.x - v.y * e.y;
-      im += v.x * e.y + v.y * e.x;
+  Q *Es = reinterpret_cast<Q *>(smem_raw);  // [N][JB]
+  const long b = blockIdx.z;
+  const int a = blockIdx.y, c = blockIdx.x * blockDim.x * CB + threadIdx.x, tid = threadIdx.x;
+  const P2 *src = reinterpret_cast<const P2 *>(in) + (b * A + a) * (long)N * C + c;
+  const C2<T> *eb = E + b * es + (long)axis * N * nt;
+  P2 *dst = reinterpret_cast<P2 *>(out) + (b * A + a) * (long)nt * C + c;
+  int off[CB];  // a column past the end reads the thread's first
+#pragma unroll
+  for (int u = 0; u < CB; ++u) off[u] = c + u * (int)blockDim.x < C ? u * blockDim.x : 0;
+  for (int j0 = 0; j0 < nt; j0 += JB) {
+    __syncthreads();
+    for (int t = tid; t < N * JB; t += blockDim.x) {
+      const int k = t / JB, j = j0 + t % JB;
+      const C2<T> e = j < nt ? eb[k * nt + j] : C2<T>{T(0), T(0)};
+      Es[t] = Q{e.x, e.x, -e.y, e.y};
     }
-    dstb[(long)j * C + c0 + c] = C2<T>{re, im};
+    __syncthreads();
+    if (c >= C) continue;
+    P2 acc[CB][JB];
+#pragma unroll
+    for (int u = 0; u < CB; ++u)
+#pragma unroll
+      for (int j = 0; j < JB; ++j) acc[u][j].x = acc[u][j].y = T(0);
+    constexpr int U = 4;
+    P2 nx[U][CB];
+    auto load = [&](int k0) {
+#pragma unroll
+      for (int q = 0; q < U; ++q)
+#pragma unroll
+        for (int u = 0; u < CB; ++u)
+          if (k0 + q < N) nx[q][u] = src[(long)(k0 + q) * C + off[u]];
+    };
+    load(0);
+    for (int k0 = 0; k0 < N; k0 += U) {
+      P2 v[U][CB];
+#pragma unroll
+      for (int q = 0; q < U; ++q)
+#pragma unroll
+        for (int u = 0; u < CB; ++u) v[q][u] = nx[q][u];
+      load(k0 + U);
+#pragma unroll
+      for (int q = 0; q < U; ++q) {
+        if (k0 + q >= N) break;
+#pragma unroll
+        for (int j = 0; j < JB; ++j) {
+          const Q e = Es[(k0 + q) * JB + j];
+#pragma unroll
+          for (int u = 0; u < CB; ++u) acc[u][j] = cmac(acc[u][j], v[q][u], e);
+        }
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < CB; ++u)
+      if (u == 0 || off[u])
+#pragma unroll
+        for (int j = 0; j < JB; ++j)
+          if (j0 + j < nt) dst[(long)(j0 + j) * C + off[u]] = acc[u][j];
   }
 }
 
@@ -359,7 +583,7 @@ k_idft_mid(const C2<T> *__restrict__ in, C2<T> *__restrict__ out, const C2<T> *_
 template <typename T>
 __global__ void __launch_bounds__(256)
 k_idft_x(const C2<T> *__restrict__ Y, T *__restrict__ CC, const C2<T> *__restrict__ E, int N,
-         int nt, int rows, T scale) {
+         int nt, int rows, T scale, long es) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   constexpr int ROWS = 8;
   C2<T> *ys = reinterpret_cast<C2<T> *>(smem_raw);  // [ROWS][N]
@@ -372,7 +596,7 @@ k_idft_x(const C2<T> *__restrict__ Y, T *__restrict__ CC, const C2<T> *__restric
     const int r = idx / N;
     ys[idx] = r0 + r < rows ? yb[(long)r0 * N + idx] : C2<T>{T(0), T(0)};
   }
-  const C2<T> *eb = E + (b * 3) * (long)N * nt;
+  const C2<T> *eb = E + b * es;
   for (int idx = tid; idx < N * nt; idx += NT) Es[idx] = eb[idx];
   __syncthreads();
   for (int o = tid; o < ROWS * nt; o += NT) {
@@ -479,26 +703,39 @@ static cudaError_t idft_grid(const Plan &p, int B, int nt, const double *org, in
                              cudaStream_t st) {
   const int N = p.N;
   const long N2 = (long)N * N;
-  const long nE = (long)B * 3 * N * nt;
-  k_idft_factors<T><<<(unsigned)((nE + 255) / 256), 256, 0, st>>>((C2<T> *)w.E, N, nt, B, org, j0, den);
-  // z stage: X[b][kz][ky kx] -> Y1[b][tz][ky kx]
+  // the integer window has the same factors for every particle
+  const int nb = org ? B : 1;
+  const long es = org ? 3L * N * nt : 0;
+  k_idft_factors<T><<<3 * nb * ((N * nt + 255) / 256), 256, 0, st>>>((C2<T> *)w.E, N, nt, org, j0, den);
+  // z stage: X[b][kz][ky kx] -> Y1[b][tz][ky kx], then y stage: Y1[b][tz][ky][kx]
+  // -> Y2[b][tz][ty][kx]; the grid points per pass over a column: the fewest passes
+  // of at most 16 (8 in FP64), rounded up to 4
   const size_t cs = sizeof(C2<T>);
-  int TC = 64;
-  while (TC > 8 && cs * ((size_t)N * TC + (size_t)N * nt) > 96 * 1024) TC /= 2;
-  size_t smem = cs * ((size_t)N * TC + (size_t)N * nt);
-  cudaFuncSetAttribute(k_idft_mid<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  k_idft_mid<T><<<dim3((unsigned)((N2 + TC - 1) / TC), B), 256, smem, st>>>(
-      (const C2<T> *)w.Z, (C2<T> *)w.Y1, (const C2<T> *)w.E, N, nt, 1, N2, TC, 2);
-  // y stage: Y1[b][tz][ky][kx] -> Y2[b][tz][ty][kx]
-  int TCy = TC < N ? TC : N;
-  k_idft_mid<T><<<dim3((unsigned)(nt * ((N + TCy - 1) / TCy)), B), 256, smem, st>>>(
-      (const C2<T> *)w.Y1, (C2<T> *)w.Y2, (const C2<T> *)w.E, N, nt, nt, N, TCy, 1);
+  const int most = sizeof(T) == 8 ? 8 : 16, passes = (nt + most - 1) / most;
+  const int JB = ((nt + passes - 1) / passes + 3) / 4 * 4;
+  auto pick = [&](auto cb) {
+    constexpr int CB = decltype(cb)::value;
+    if constexpr (sizeof(T) == 4)
+      if (JB > 8) return JB == 12 ? k_idft_mid<T, 12, CB> : k_idft_mid<T, 16, CB>;
+    return JB == 4 ? k_idft_mid<T, 4, CB> : k_idft_mid<T, 8, CB>;
+  };
+  // two columns per thread in the z stage, which has N^2 of them per volume; rows of
+  // the y stage are short, one column keeps their CTAs many (11 points: 23 against 33 us)
+  auto midz = pick(std::integral_constant<int, 2>{}), midy = pick(std::integral_constant<int, 1>{});
+  const size_t smem = 2 * cs * (size_t)N * JB;
+  cudaFuncSetAttribute(midz, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaFuncSetAttribute(midy, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const int ty = N <= 64 ? 64 : 128;
+  midz<<<dim3((unsigned)((N2 + 255) / 256), 1, B), 128, smem, st>>>(
+      (const C2<T> *)w.Z, (C2<T> *)w.Y1, (const C2<T> *)w.E, N, nt, 1, (int)N2, 2, es);
+  midy<<<dim3((N + ty - 1) / ty, nt, B), ty, smem, st>>>(
+      (const C2<T> *)w.Y1, (C2<T> *)w.Y2, (const C2<T> *)w.E, N, nt, nt, N, 1, es);
   // x stage: Y2[b][tz ty][kx] -> CC[b][tz ty][tx]
   const int rows = nt * nt;
   size_t smx = cs * (8 * (size_t)N + (size_t)N * nt);
   cudaFuncSetAttribute(k_idft_x<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smx);
   k_idft_x<T><<<dim3((rows + 7) / 8, B), 256, smx, st>>>(
-      (const C2<T> *)w.Y2, (T *)w.CC, (const C2<T> *)w.E, N, nt, rows, T(1.0 / ((double)N2 * N)));
+      (const C2<T> *)w.Y2, (T *)w.CC, (const C2<T> *)w.E, N, nt, rows, T(1.0 / ((double)N2 * N)), es);
   k_cc_argmax<T><<<B, 256, 0, st>>>((const T *)w.CC, nt, org, j0, den, edge, flag_mode, R, t_out,
                                     tau_out, cc_out, flags);
   return cudaGetLastError();
@@ -510,27 +747,40 @@ cudaError_t launch_shift_search(const Plan &p, const float *f, const float *u, i
                                 double *t, double *tau, double *cc, int *flags, cudaStream_t st) {
   if (B <= 0) return cudaSuccess;
   const int N = p.N;
-  const long N2 = (long)N * N, N3 = N2 * N;
+  const long N2 = (long)N * N;
   FftDesc fd;
   fd.N = N;
   fd.npass = p.fft_npass;
   for (int q = 0; q < 16; ++q) fd.radix[q] = p.fft_radix[q];
   const size_t cs = sizeof(C2<T>);
-  // lines per CTA: about 4096 elements (a whole 64 x 64 plane), at least 16
-  // columns for the strided passes so their rows stay coalesced
-  const int NB0 = N * N <= 4096 ? N : (4096 / N > 0 ? 4096 / N : 1);
-  const int NB = N <= 64 ? N : (4096 / N > 16 ? 4096 / N : 16);
-  size_t sm0 = cs * 2 * (size_t)NB0 * (N + 1), sm1 = cs * 2 * (size_t)NB * (N + 1);
-  size_t smax = sm0 > sm1 ? sm0 : sm1;
-  cudaFuncSetAttribute(k_fft_axis<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smax);
   C2<T> *Z = (C2<T> *)w.Z;
   const C2<T> *tw = (const C2<T> *)p.fft_tw;
-  const T fwd = T(-1);
-  k_fft_axis<T><<<dim3((unsigned)((N2 + NB0 - 1) / NB0), B), 256, sm0, st>>>(Z, f, u, 0, fd, tw, NB0, fwd);
-  const unsigned tiles = (unsigned)(N * ((N + NB - 1) / NB));
-  k_fft_axis<T><<<dim3(tiles, B), 256, sm1, st>>>(Z, nullptr, nullptr, 1, fd, tw, NB, fwd);
-  k_fft_axis<T><<<dim3(tiles, B), 256, sm1, st>>>(Z, nullptr, nullptr, 2, fd, tw, NB, fwd);
-  k_cross_spectrum<T><<<dim3((unsigned)((N3 + 255) / 256), B), 256, 0, st>>>(Z, N);
+  // planes of which two buffers fit an SM (N <= 112 in FP32, 79 in FP64) are transformed
+  // whole; larger ones a direction at a time
+  const size_t plane = cs * (2 * (size_t)N * (N | 1) + N);
+  if (plane <= 200 * 1024) {
+    cudaFuncSetAttribute(k_fft_plane<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)plane);
+    k_fft_plane<T><<<dim3(N, B), 256, plane, st>>>(Z, f, u, fd, tw);
+  } else {
+    // rows, then columns (at least 16, so their rows stay coalesced), about 4096
+    // elements per CTA
+    const int NB0 = 4096 / N > 0 ? 4096 / N : 1, NB = 4096 / N > 16 ? 4096 / N : 16;
+    const size_t sm0 = cs * (2 * (size_t)NB0 * (N | 1) + N), sm1 = cs * (2 * (size_t)NB * (N | 1) + N);
+    cudaFuncSetAttribute(k_fft_axis<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)(sm0 > sm1 ? sm0 : sm1));
+    k_fft_axis<T><<<dim3((unsigned)((N2 + NB0 - 1) / NB0), B), 256, sm0, st>>>(Z, f, u, 0, fd, tw, NB0);
+    k_fft_axis<T><<<dim3((unsigned)(N * ((N + NB - 1) / NB)), B), 256, sm1, st>>>(Z, nullptr, nullptr, 1,
+                                                                               fd, tw, NB);
+  }
+  // columns of the z transform per CTA: 128-byte rows while four buffers of them
+  // leave two CTAs on an SM
+  int NBz = 128 / (int)cs;
+  while (NBz > 1 && cs * (4 * (size_t)NBz + 1) * N > 112 * 1024) NBz /= 2;
+  const size_t smz = cs * (4 * (size_t)NBz + 1) * N;
+  cudaFuncSetAttribute(k_fft_cross<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smz);
+  const int nself = N % 2 ? 1 : 2, npair = (N - nself) / 2;
+  const unsigned zt = nself * ((N / 2 + NBz) / NBz) + npair * ((N + NBz - 1) / NBz);
+  k_fft_cross<T><<<dim3(zt, B), 128, smz, st>>>(Z, fd, tw, NBz);
   cudaError_t e;
   // integer window [-m, m]^3
   const int nw = 2 * max_shift + 1;
