@@ -28,6 +28,7 @@
 #include <algorithm>
 #include <float.h>
 #include <limits.h>
+#include <cooperative_groups.h>
 #include "internal.cuh"
 
 namespace matcha {
@@ -768,6 +769,8 @@ size_t soft_warps_smem(const Plan &p) {
          4 * (capc + 32 + 4) + 16;
 }
 
+constexpr int SOFT_SPLIT_MOST = 9;  // CTAs of a cluster that shares a particle, at most
+
 // Register-tiled chunked variant (32-bit plans, soft_n % 4 == 0): the pass
 // structure of k_soft_chunk (KB new beta slices per pass into a ring of KB+2,
 // then the local maxima of KB slices), with every phase cut into exactly as
@@ -786,15 +789,24 @@ size_t soft_warps_smem(const Plan &p) {
 // stage loops unroll); local maxima that cannot enter the best-P list (once
 // it holds P_b entries, those that do not precede its last one) are not
 // queued for the merge.
-template <int KB, int L0, int ns>
-__global__ void __launch_bounds__(384, 2)
-k_soft_tile(const float *__restrict__ c, long nc, const int *__restrict__ pair_base,
+//
+// CL > 1: the beta slices of a particle are split over a cluster of CL CTAs, each
+// with ns / CL of them and the slice before and after (recomputed); the first CTA
+// merges the others' best-P lists.  The order of candidates is total, so the result
+// is the same.
+template <int KB, int L0, int ns, int CL>
+__device__ __forceinline__ void
+soft_tile(const float *__restrict__ c, long nc, const int *__restrict__ pair_base,
             const float *__restrict__ soft_d, const int *__restrict__ pair_off0, long nc0,
             const float *__restrict__ tw, int P_max, const int *__restrict__ P_per,
             float *__restrict__ grid_out, int *__restrict__ idx_out, double *__restrict__ euler_out,
             double *__restrict__ score_out, int *__restrict__ n_cand_out) {
   constexpr int NR = KB + 2;
-  const long b = blockIdx.x;
+  static_assert(ns % CL == 0 && ns / CL % KB == 0, "whole passes per CTA");
+  constexpr int NB = CL > 1 ? KB + 2 : KB + 1;  // slices of a CTA's first pass
+  const long b = CL > 1 ? blockIdx.x / CL : blockIdx.x;
+  const int rank = CL > 1 ? blockIdx.x % CL : 0;
+  const int ks = rank * (ns / CL), ke = ks + ns / CL;
   static_assert(ns % 4 == 0, "gamma quads");
   constexpr int W = 2 * L0 + 1, M1 = L0 + 1, np0 = M1 * M1, n2 = ns * ns, q4 = ns / 4;
   const int tid = threadIdx.x, NT = blockDim.x;
@@ -803,12 +815,12 @@ k_soft_tile(const float *__restrict__ c, long nc, const int *__restrict__ pair_b
   auto al4 = [](long x) { return (x + 3) & ~3L; };
   float *ring = reinterpret_cast<float *>(smem_raw);  // [NR][n2]
   float *mx = ring + al4(NR * n2);                     // [NR][n2] 3x3 (alpha, gamma) maxima
-  float *G = mx + al4(NR * n2);                        // [KB+1][2 M1][ns]: rows (Re, Im) of G_m
-  float *Eg = G + al4((KB + 1) * 2 * M1 * ns);         // [W][q4][12]: cos, sin, -sin of 4 gammas
+  float *G = mx + al4(NR * n2);                        // [NB][2 M1][ns]: rows (Re, Im) of G_m
+  float *Eg = G + al4(NB * 2 * M1 * ns);               // [W][q4][12]: cos, sin, -sin of 4 gammas
   float *Ad = Eg + al4(W * q4 * 12);                   // [2 M1][ns][2]: (a, a)
   float *cst = Ad + al4(2 * M1 * ns * 2);              // [nc0][4] staged c, l <= L0
-  const long sdn = al4(max((long)(KB + 1) * M1 * W * 4, 2L * capc));
-  float *Sd = cst + al4(4 * nc0);                      // [KB+1][M1][W][4]: (Re, Re, Im, Im)
+  const long sdn = al4(max((long)NB * M1 * W * 4, 2L * capc));
+  float *Sd = cst + al4(4 * nc0);                      // [NB][M1][W][4]: (Re, Re, Im, Im)
   float *cv = Sd;                                      // [capc] candidates (alias of Sd)
   int *ci = reinterpret_cast<int *>(Sd + capc);        // [capc]
   float *rv = Sd + sdn;                                // [32]
@@ -862,8 +874,8 @@ k_soft_tile(const float *__restrict__ c, long nc, const int *__restrict__ pair_b
   if (tid < 32) { rv[tid] = 0; ri[tid] = INT_MAX; }
   if (tid == 0) counters[1] = 0;
   __syncthreads();
-  int done = 0;  // slices [0, done) computed
-  for (int k0 = 0; k0 < ns; k0 += KB) {
+  int done = max(ks - 1, 0);  // slices below computed, or not needed
+  for (int k0 = ks; k0 < ke; k0 += KB) {
     const int hi = min(ns, k0 + KB + 1), ka = done, nk = hi - ka;
     // phase 1: beta transform of slices ka..hi-1 into the rows m >= 0 of S
     for (int t = tid; t < nk * np0; t += NT) {
@@ -1066,6 +1078,38 @@ k_soft_tile(const float *__restrict__ c, long nc, const int *__restrict__ pair_b
     }
     __syncthreads();
   }
+  if (CL > 1) {
+    namespace cg = cooperative_groups;
+    cg::cluster_group cl = cg::this_cluster();
+    cl.sync();
+    if (rank == 0 && tid < 32) {
+      const int lane = tid;
+      float myv = rv[lane];
+      int myi = ri[lane];
+      int kept = counters[1];
+      for (int q = 1; q < CL; ++q) {
+        const float ov = cl.map_shared_rank(rv, q)[lane];
+        const int oi = cl.map_shared_rank(ri, q)[lane], cnt = cl.map_shared_rank(counters, q)[1];
+        for (int e = 0; e < cnt; ++e) {
+          const float v = __shfl_sync(0xffffffffu, ov, e);
+          const int i = __shfl_sync(0xffffffffu, oi, e);
+          const bool before = lane < kept && precedes(myv, myi, v, i);
+          const int pos = __popc(__ballot_sync(0xffffffffu, before));
+          if (pos >= Pb) break;  // nor do the entries after it
+          const float upv = __shfl_up_sync(0xffffffffu, myv, 1);
+          const int upi = __shfl_up_sync(0xffffffffu, myi, 1);
+          if (lane > pos) { myv = upv; myi = upi; }
+          if (lane == pos) { myv = v; myi = i; }
+          kept = min(kept + 1, Pb);
+        }
+      }
+      rv[lane] = myv;
+      ri[lane] = myi;
+      if (lane == 0) counters[1] = kept;
+    }
+    cl.sync();  // the lists were read
+    if (rank) return;
+  }
   const int kept = counters[1];
   for (int r = tid; r < P_max; r += NT) {
     long o = b * P_max + r;
@@ -1086,15 +1130,36 @@ k_soft_tile(const float *__restrict__ c, long nc, const int *__restrict__ pair_b
   if (tid == 0) n_cand_out[b] = kept;
 }
 
+template <int KB, int L0, int ns>
+__global__ void __launch_bounds__(384, 2)
+k_soft_tile(const float *__restrict__ c, long nc, const int *__restrict__ pair_base,
+            const float *__restrict__ soft_d, const int *__restrict__ pair_off0, long nc0,
+            const float *__restrict__ tw, int P_max, const int *__restrict__ P_per,
+            float *__restrict__ grid_out, int *__restrict__ idx_out, double *__restrict__ euler_out,
+            double *__restrict__ score_out, int *__restrict__ n_cand_out) {
+  soft_tile<KB, L0, ns, 1>(c, nc, pair_base, soft_d, pair_off0, nc0, tw, P_max, P_per, grid_out, idx_out,
+                           euler_out, score_out, n_cand_out);
+}
+template <int KB, int L0, int ns, int CL>
+__global__ void __launch_bounds__(CL == SOFT_SPLIT_MOST ? 512 : 384, CL == SOFT_SPLIT_MOST ? 1 : 2)
+k_soft_split(const float *__restrict__ c, long nc, const int *__restrict__ pair_base,
+             const float *__restrict__ soft_d, const int *__restrict__ pair_off0, long nc0,
+             const float *__restrict__ tw, int P_max, const int *__restrict__ P_per,
+             float *__restrict__ grid_out, int *__restrict__ idx_out, double *__restrict__ euler_out,
+             double *__restrict__ score_out, int *__restrict__ n_cand_out) {
+  soft_tile<KB, L0, ns, CL>(c, nc, pair_base, soft_d, pair_off0, nc0, tw, P_max, P_per, grid_out, idx_out,
+                            euler_out, score_out, n_cand_out);
+}
+
 constexpr int TILE_KB = 4;
 
 // Shared memory of k_soft_tile (the layout carved at its start).
-size_t soft_tile_smem(const Plan &p) {
+size_t soft_tile_smem(const Plan &p, int extra = 0) {  // extra: 1 for CL > 1
   auto al4 = [](size_t x) { return (x + 3) & ~size_t(3); };
   const size_t W = 2 * p.L0 + 1, M1 = p.L0 + 1, ns = p.ns, n2 = ns * ns, q4 = ns / 4;
   const size_t capc = (size_t)TILE_KB * ((ns + 1) / 2) * ((ns + 1) / 2);
-  const size_t sdn = al4(std::max((TILE_KB + 1) * M1 * W * 4, 2 * capc));
-  return 4 * (2 * al4((TILE_KB + 2) * n2) + al4((TILE_KB + 1) * 2 * M1 * ns) + al4(W * q4 * 12) +
+  const size_t sdn = al4(std::max((TILE_KB + 1 + extra) * M1 * W * 4, 2 * capc));
+  return 4 * (2 * al4((TILE_KB + 2) * n2) + al4((TILE_KB + 1 + extra) * 2 * M1 * ns) + al4(W * q4 * 12) +
               al4(2 * M1 * ns * 2) + al4(4 * (size_t)p.nc0) + sdn + 32 + 32 + 4);
 }
 
@@ -1169,12 +1234,28 @@ cudaError_t launch_soft(const Plan &p, const T *c, int B, const int *P_per, T *g
   }
   // the register-tiled kernel unless another was chosen (bit-identical to the chunked one)
   if (sizeof(T) == 4 && (p.tune_soft == 0 || p.tune_soft == 3) && soft_tile_ok(p)) {
-    const size_t smem = soft_tile_smem(p);
-    cudaFuncSetAttribute(k_soft_tile<TILE_KB, 8, 36>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k_soft_tile<TILE_KB, 8, 36><<<B, soft_tile_threads(p), smem, st>>>(
-        (const float *)c, p.nc, p.pair_base, (const float *)p.soft_d, p.pair_off0,
-        p.nc0, (const float *)p.soft_tw, p.P, P_per, (float *)grid, idx, euler, score, n_cand);
-    return cudaGetLastError();
+    // a particle over nine CTAs (a pass each) while each has an SM (1 particle: 82 us on
+    // one CTA, 24), over three while two share one (96 particles: 93 us, 62)
+    const int CL = 9L * B <= p.sms ? SOFT_SPLIT_MOST : 3L * B <= 2L * p.sms ? 3 : 1;
+    const size_t smem = soft_tile_smem(p, CL > 1);
+    auto kern = CL == 9 ? k_soft_split<TILE_KB, 8, 36, SOFT_SPLIT_MOST>
+              : CL == 3 ? k_soft_split<TILE_KB, 8, 36, 3> : k_soft_tile<TILE_KB, 8, 36>;
+    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (CL > 8) cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)B * CL);
+    cfg.blockDim = dim3(CL == 9 ? 512 : soft_tile_threads(p));
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = CL;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = CL > 1;
+    return cudaLaunchKernelEx(&cfg, kern, (const float *)c, p.nc, p.pair_base, (const float *)p.soft_d,
+                              p.pair_off0, (long)p.nc0, (const float *)p.soft_tw, p.P, P_per, (float *)grid,
+                              idx, euler, score, n_cand);
   }
   {
     size_t smem = soft_chunk_smem(p, sizeof(T));
