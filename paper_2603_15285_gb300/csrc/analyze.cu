@@ -168,16 +168,21 @@ constexpr int ANALYZE_THREADS = 192;
 // CTAs per SM) or spill under a four-CTA bound, and both measure slower
 constexpr int GATHER_BATCH = 2;
 
+struct TexPair { TexArgs of[2]; };
 template <typename T, int G, bool TEX>
 __global__ void __launch_bounds__(ANALYZE_THREADS)
-k_analyze2(const float *__restrict__ vols, int N, int S, int L,
+k_analyze2(const float *__restrict__ vols, int B0, const float *__restrict__ vols2, int N, int S, int L,
            const double *__restrict__ rs, const double *__restrict__ xj, const T *__restrict__ phi_cs,
            const T *__restrict__ dcs, int Mp, int Qf, int Mq, const T *__restrict__ ptabT,
            const int *__restrict__ leg, const T *__restrict__ ring, T *__restrict__ out,
-           const __grid_constant__ TexArgs ta) {
+           T *__restrict__ out2, const __grid_constant__ TexPair ta) {
   constexpr int GB = GATHER_BATCH;
   const int s0 = blockIdx.x * G;
-  const long b = blockIdx.y;
+  // two batches (particles and templates) share a launch: volumes b >= B0 are the
+  // second's
+  const bool second = (int)blockIdx.y >= B0;
+  const long b = second ? blockIdx.y - B0 : blockIdx.y;
+  if (second) { vols = vols2; out = out2; }
   const int Gs = G;  // the launcher picks G dividing S
   const int nt = L + 1, np = 2 * L + 2, half = np / 2, K1 = half - 1;
   const int nlm = (L + 1) * (L + 2) / 2;
@@ -210,9 +215,9 @@ k_analyze2(const float *__restrict__ vols, int N, int S, int L,
   cudaTextureObject_t tob = 0;
   float yoff = 0.f;  // first row of this volume in its texture view
   if (TEX) {
-    const int run = (int)(b / ta.vpt);
-    tob = ta.t[run];
-    yoff = (float)((b - (long)run * ta.vpt) * NN);
+    const int vpt = ta.of[second].vpt, run = (int)b / vpt;
+    tob = ta.of[second].t[run];
+    yoff = (float)((b - (long)run * vpt) * NN);
   }
   // trilinear combination of the two gathered planes (components: x (i, j+1),
   // y (i+1, j+1), z (i+1, j), w (i, j)) at cell offsets (tx, ty, tz)
@@ -512,37 +517,89 @@ size_t analyze2_smem(const Plan &p, int G) {
                       2 * (size_t)Rp * p.Mp + 2 * (size_t)p.np);
 }
 
+// Shells per CTA and shared-memory carve-out (percent; -1: the driver's, the smallest
+// for the most CTAs) of the shell-group kernel.  The gathers live on L1, which is what
+// the carve-out leaves.
+//   FP32, N >= 128 and four CTAs of two shells take more than 164 KB: neighbouring
+//     samples of a ring are voxels apart and share few sectors.  One shell per CTA, and
+//     CTAs only as far as 164 KB of shared memory go (24 volumes of 200^3, 40 shells,
+//     L_J = 40: 206 us with two shells, 100 with one; 60 of 128^3, L_J = 48: 242 with
+//     two, 257 with one on all 228 KB, 216 on 164; up to L_J = 28 two are as fast).  The
+//     limit helps single shells from N = 88 on (64 of 90^3, L_J = 48: 332 us without,
+//     235 with it) while three CTAs fit, two on the larger boxes (64 of 96^3, L_J =
+//     56: 321 without, 400 with it; of 130^3: 593, 440).
+//   FP32, smaller boxes: two shells share the tables' reads (600 volumes of 64^3, L_J =
+//     32: 382 us against 477), unless four CTAs no longer fit an SM and the waves of
+//     single shells are shorter (600 of 64^3, L_J = 40: 737 us with two, 678 with one;
+//     200 of 96^3: 425, 328).
+//   FP64: bound by its pipe, two shells (40 volumes of 64^3: 460 us, 495 with one).
+struct AnalyzeShape { int G, carve; };
 template <typename T>
-cudaError_t launch_analyze(const Plan &p, const float *vols, int B, T *coef, cudaStream_t st) {
+static AnalyzeShape analyze_shape(const Plan &p, long volumes) {
+  auto cost = [&](int g) { return analyze2_smem<T>(p, g) + 1024; };  // a CTA's, with the system's
+  const bool large = sizeof(T) == 4 && p.N >= 128 && 4 * cost(2) > 164 * 1024;
+  int G = p.tune_shells;
+  if (G <= 0) {
+    G = 2;
+    if (sizeof(T) == 4 && cost(2) > 49 * 1024) {
+      auto rounds = [&](int g) {
+        const long fit = std::max<long>(1, std::min<long>(4, 227 * 1024 / cost(g))) * p.sms;
+        return (volumes * (p.S / g) + fit - 1) / fit;
+      };
+      if (rounds(1) < 2 * rounds(2)) G = 1;
+    }
+    // (on 128^3 a single wave of double shells is still as fast)
+    if (large && (p.N >= 144 || volumes * (p.S / 2) > 4L * p.sms)) G = 1;
+  }
+  G = G >= 8 ? 8 : G >= 4 ? 4 : G >= 2 ? 2 : 1;
+  while (G > 1 && (p.S % G != 0 || analyze2_smem<T>(p, G) > 100 * 1024)) G >>= 1;
+  // three CTAs on 164 KB, or two where the box is large
+  const bool cap = sizeof(T) == 4 && G == 1 && p.N >= 88 && cost(1) <= (p.N > 128 ? 82 : 54) * 1024;
+  return {G, cap ? 71 : -1};
+}
+
+// Analyses B volumes into coef and, in the same launch where it can, B2 into coef2.
+template <typename T>
+cudaError_t launch_analyze(const Plan &p, const float *vols, int B, T *coef, cudaStream_t st,
+                           const float *vols2, int B2, T *coef2) {
+  if (B == 0 && B2 > 0) return launch_analyze<T>(p, vols2, B2, coef2, st, nullptr, 0, nullptr);
   if (B == 0) return cudaSuccess;
   {
-    // shells per CTA: a divisor of S in {8, 4, 2, 1} whose shared memory fits;
-    // 2 unless the plan was autotuned (matcha_plan_autotune)
-    int G = p.tune_shells > 0 ? p.tune_shells : 2;
-    G = G >= 8 ? 8 : G >= 4 ? 4 : G >= 2 ? 2 : 1;
-    while (G > 1 && (p.S % G != 0 || analyze2_smem<T>(p, G) > 100 * 1024)) G >>= 1;
+    const AnalyzeShape sh = analyze_shape<T>(p, (long)B + B2);
+    const int G = sh.G;
     size_t smem = analyze2_smem<T>(p, G);
-    if (smem <= 200 * 1024) {
+    if (smem <= 200 * 1024 && (long)B + B2 <= 65535) {
       std::lock_guard<std::mutex> lock(p.tex_mu);
-      TexArgs ta;
-      const bool tex = texture_views(p, vols, B, st, ta);
+      TexPair tp;
+      const bool tex = texture_views(p, vols, B, st, tp.of[0]);
+      const bool tex2 = B2 > 0 ? texture_views(p, vols2, B2, st, tp.of[1]) : tex;
       auto pick = [&](auto tag) {
         constexpr bool X = decltype(tag)::value;
         return G == 8 ? k_analyze2<T, 8, X> : G == 4 ? k_analyze2<T, 4, X>
              : G == 2 ? k_analyze2<T, 2, X> : k_analyze2<T, 1, X>;
       };
-      auto kern = tex ? pick(std::true_type{}) : pick(std::false_type{});
-      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
       // 192 threads: six warps per CTA keep four CTAs resident per SM
       // (measured 1.27 ms per 1,024 batch64 particles against 1.41 with 256
       // threads and 1.59 with 128)
-      kern<<<dim3(p.S / G, B), ANALYZE_THREADS, smem, st>>>(vols, p.N, p.S, p.LJ, p.rs, p.xj,
-                                                (const T *)p.phi_cs, (const T *)p.dft_cs, p.Mp,
-                                                p.Qf, p.Mq, (const T *)p.ptab_leg, p.leg_lm,
-                                                (const T *)p.ring,
-                                                coef, ta);
-      return cudaGetLastError();
+      auto run = [&](bool x, const float *v, int n, T *o, int n2) {
+        auto kern = x ? pick(std::true_type{}) : pick(std::false_type{});
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, sh.carve);
+        kern<<<dim3(p.S / G, n + n2), ANALYZE_THREADS, smem, st>>>(
+            v, n, vols2, p.N, p.S, p.LJ, p.rs, p.xj, (const T *)p.phi_cs, (const T *)p.dft_cs, p.Mp, p.Qf,
+            p.Mq, (const T *)p.ptab_leg, p.leg_lm, (const T *)p.ring, o, coef2, tp);
+        return cudaGetLastError();
+      };
+      if (tex == tex2) return run(tex, vols, B, coef, B2);
+      const cudaError_t e = run(tex, vols, B, coef, 0);
+      if (e != cudaSuccess) return e;
+      tp.of[0] = tp.of[1];
+      return run(tex2, vols2, B2, coef2, 0);
     }
+  }
+  if (B2 > 0) {
+    const cudaError_t e = launch_analyze<T>(p, vols, B, coef, st, nullptr, 0, nullptr);
+    return e != cudaSuccess ? e : launch_analyze<T>(p, vols2, B2, coef2, st, nullptr, 0, nullptr);
   }
   // rings per batch: as many as fit next to F (all of them when they do)
   const size_t fixed = 2 * (size_t)p.nt * (p.LJ + 1) + 2 * (size_t)p.np;
@@ -562,7 +619,9 @@ bool analyze_shells_ok(const Plan &p, int G) {
   return p.fp64 ? analyze2_smem<double>(p, G) <= 100 * 1024 : analyze2_smem<float>(p, G) <= 100 * 1024;
 }
 
-template cudaError_t launch_analyze<float>(const Plan &, const float *, int, float *, cudaStream_t);
-template cudaError_t launch_analyze<double>(const Plan &, const float *, int, double *, cudaStream_t);
+template cudaError_t launch_analyze<float>(const Plan &, const float *, int, float *, cudaStream_t,
+                                           const float *, int, float *);
+template cudaError_t launch_analyze<double>(const Plan &, const float *, int, double *, cudaStream_t,
+                                            const float *, int, double *);
 
 }  // namespace matcha

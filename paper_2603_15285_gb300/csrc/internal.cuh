@@ -144,7 +144,8 @@ int ball_tables(int L, int S, double R, double Lam, const double *r, const doubl
 
 // Kernel launchers; each returns cudaGetLastError() after its launches.
 template <typename T>
-cudaError_t launch_analyze(const Plan &p, const float *vols, int B, T *coef, cudaStream_t st);
+cudaError_t launch_analyze(const Plan &p, const float *vols, int B, T *coef, cudaStream_t st,
+                           const float *vols2 = nullptr, int B2 = 0, T *coef2 = nullptr);
 template <typename T>
 cudaError_t launch_correlate(const Plan &p, const T *f, const T *h, int B, int hstride, T *c,
                              cudaStream_t st);

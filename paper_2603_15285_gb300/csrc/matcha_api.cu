@@ -465,8 +465,15 @@ static matcha_status align_range(matcha_plan plan, const float *particles, const
   matcha_status s;
   {
     Range r("a1+a2 analysis");
-    if ((s = matcha_analyze(plan, particles, B, w.f, stream))) return s;
-    if (!h_ready && (s = matcha_analyze(plan, templates, Bt, w.h, stream))) return s;
+    if (B < 0 || B > 65535 || (B > 0 && (!particles || !w.f)))
+      return B > 65535 ? MATCHA_ERR_UNSUPPORTED : MATCHA_ERR_INVALID_ARG;
+    if (!h_ready && Bt > 0 && (!templates || !w.h)) return MATCHA_ERR_INVALID_ARG;
+    cudaStream_t st = (cudaStream_t)stream;
+    const int B2 = h_ready ? 0 : Bt;
+    const cudaError_t e =
+        p->fp64 ? launch_analyze<double>(*p, particles, B, (double *)w.f, st, templates, B2, (double *)w.h)
+                : launch_analyze<float>(*p, particles, B, (float *)w.f, st, templates, B2, (float *)w.h);
+    if (e != cudaSuccess) return fail_cuda(e, "analyze");
   }
   {
     Range r("a3 contraction");
