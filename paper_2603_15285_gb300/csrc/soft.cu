@@ -251,6 +251,37 @@ k_soft_stream(const T *__restrict__ c, long nc, int L0, int ns, const int *__res
 // once (three phases over all of them) into a ring of KB+2 slices, then tests
 // the local maxima of KB slices and merges them, so each barrier separates
 // KB times more independent work than the one-slice version.
+// The best-P lists of a cluster's CTAs (sorted; the counters' second entry: their
+// length) merged into the first one's, by its first warp.  The order is total, so the
+// split leaves no trace.
+template <typename T>
+__device__ __forceinline__ void merge_lists(cooperative_groups::cluster_group &cl, int CL, T *rv, int *ri,
+                                            int *counters, int Pb) {
+  const int lane = threadIdx.x;
+  T myv = rv[lane];
+  int myi = ri[lane];
+  int kept = counters[1];
+  for (int q = 1; q < CL; ++q) {
+    const T ov = cl.map_shared_rank(rv, q)[lane];
+    const int oi = cl.map_shared_rank(ri, q)[lane], cnt = cl.map_shared_rank(counters, q)[1];
+    for (int e = 0; e < cnt; ++e) {
+      const T v = __shfl_sync(0xffffffffu, ov, e);
+      const int i = __shfl_sync(0xffffffffu, oi, e);
+      const bool before = lane < kept && precedes(myv, myi, v, i);
+      const int pos = __popc(__ballot_sync(0xffffffffu, before));
+      if (pos >= Pb) break;  // nor do the entries after it
+      const T upv = __shfl_up_sync(0xffffffffu, myv, 1);
+      const int upi = __shfl_up_sync(0xffffffffu, myi, 1);
+      if (lane > pos) { myv = upv; myi = upi; }
+      if (lane == pos) { myv = v; myi = i; }
+      kept = min(kept + 1, Pb);
+    }
+  }
+  rv[lane] = myv;
+  ri[lane] = myi;
+  if (lane == 0) counters[1] = kept;
+}
+
 constexpr int CHUNK_THREADS = 512;
 
 template <typename T> struct Vec4;
@@ -267,9 +298,13 @@ k_soft_chunk(const T *__restrict__ c, long nc, int L0, int ns, const int *__rest
              const T *__restrict__ soft_d, const int *__restrict__ pair_off0, long nc0,
              const T *__restrict__ tw, int P_max, const int *__restrict__ P_per,
              T *__restrict__ grid_out, int *__restrict__ idx_out, double *__restrict__ euler_out,
-             double *__restrict__ score_out, int *__restrict__ n_cand_out) {
+             double *__restrict__ score_out, int *__restrict__ n_cand_out, int CL) {
   constexpr int NR = KB + 2;
-  const long b = blockIdx.x;
+  const long b = blockIdx.x / CL;
+  const int rank = blockIdx.x - (int)b * CL;
+  // this CTA's slices, whole passes; after the first CTA's, a pass that only computes
+  // the slice before them and the first one goes ahead
+  const int per = ((ns + KB - 1) / KB + CL - 1) / CL * KB, ks = min(ns, rank * per), ke = min(ns, ks + per);
   const int W = 2 * L0 + 1, np0 = (L0 + 1) * (L0 + 1), n2 = ns * ns;
   const int tid = threadIdx.x, NT = blockDim.x;
   const int capc = KB * ((ns + 1) / 2) * ((ns + 1) / 2);
@@ -329,8 +364,8 @@ k_soft_chunk(const T *__restrict__ c, long nc, int L0, int ns, const int *__rest
   if (tid < 32) { rv[tid] = 0; ri[tid] = INT_MAX; }
   if (tid == 0) counters[1] = 0;
   __syncthreads();
-  int done = 0;  // slices [0, done) computed
-  for (int k0 = 0; k0 < ns; k0 += KB) {
+  int done = max(ks - 1, 0);  // slices below computed, or not needed
+  for (int k0 = max(ks - KB, 0); k0 < ke; k0 += KB) {
     const int hi = min(ns, k0 + KB + 1), ka = done, nk = hi - ka;
     // phase 1: beta transform of slices ka..hi-1
     for (int t = tid; t < nk * np0; t += NT) {
@@ -427,6 +462,7 @@ k_soft_chunk(const T *__restrict__ c, long nc, int L0, int ns, const int *__rest
     done = hi;
     if (tid == 0) counters[0] = 0;
     __syncthreads();
+    if (k0 < ks) continue;
     const int k1 = min(ns, k0 + KB), nt_ = k1 - k0;
     if (grid_out) {
       T *go = grid_out + b * (long)ns * n2;
@@ -499,6 +535,13 @@ k_soft_chunk(const T *__restrict__ c, long nc, int L0, int ns, const int *__rest
       if (lane == 0) counters[1] = kept;
     }
     __syncthreads();
+  }
+  if (CL > 1) {
+    cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
+    cl.sync();
+    if (rank == 0 && tid < 32) merge_lists(cl, CL, rv, ri, counters, Pb);
+    cl.sync();  // the lists were read
+    if (rank) return;
   }
   const int kept = counters[1];
   for (int r = tid; r < P_max; r += NT) {
@@ -1082,31 +1125,7 @@ soft_tile(const float *__restrict__ c, long nc, const int *__restrict__ pair_bas
     namespace cg = cooperative_groups;
     cg::cluster_group cl = cg::this_cluster();
     cl.sync();
-    if (rank == 0 && tid < 32) {
-      const int lane = tid;
-      float myv = rv[lane];
-      int myi = ri[lane];
-      int kept = counters[1];
-      for (int q = 1; q < CL; ++q) {
-        const float ov = cl.map_shared_rank(rv, q)[lane];
-        const int oi = cl.map_shared_rank(ri, q)[lane], cnt = cl.map_shared_rank(counters, q)[1];
-        for (int e = 0; e < cnt; ++e) {
-          const float v = __shfl_sync(0xffffffffu, ov, e);
-          const int i = __shfl_sync(0xffffffffu, oi, e);
-          const bool before = lane < kept && precedes(myv, myi, v, i);
-          const int pos = __popc(__ballot_sync(0xffffffffu, before));
-          if (pos >= Pb) break;  // nor do the entries after it
-          const float upv = __shfl_up_sync(0xffffffffu, myv, 1);
-          const int upi = __shfl_up_sync(0xffffffffu, myi, 1);
-          if (lane > pos) { myv = upv; myi = upi; }
-          if (lane == pos) { myv = v; myi = i; }
-          kept = min(kept + 1, Pb);
-        }
-      }
-      rv[lane] = myv;
-      ri[lane] = myi;
-      if (lane == 0) counters[1] = kept;
-    }
+    if (rank == 0 && tid < 32) merge_lists(cl, CL, rv, ri, counters, Pb);
     cl.sync();  // the lists were read
     if (rank) return;
   }
@@ -1217,6 +1236,24 @@ bool soft_warps_ok(const Plan &p) {
   return !p.fp64 && soft_warps_smem<SOFT_NW>(p) <= 113 * 1024;
 }
 
+// B clusters of CL CTAs (one CTA: an ordinary launch).
+template <typename K, typename... Args>
+static cudaError_t launch_clusters(K kern, int B, int CL, int threads, size_t smem, cudaStream_t st, Args... args) {
+  if (CL > 8) cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)B * CL);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = CL;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = CL > 1;
+  return cudaLaunchKernelEx(&cfg, kern, args...);
+}
+
 template <typename T>
 cudaError_t launch_soft(const Plan &p, const T *c, int B, const int *P_per, T *grid, int *idx,
                         double *euler, double *score, int *n_cand, cudaStream_t st) {
@@ -1241,31 +1278,30 @@ cudaError_t launch_soft(const Plan &p, const T *c, int B, const int *P_per, T *g
     auto kern = CL == 9 ? k_soft_split<TILE_KB, 8, 36, SOFT_SPLIT_MOST>
               : CL == 3 ? k_soft_split<TILE_KB, 8, 36, 3> : k_soft_tile<TILE_KB, 8, 36>;
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (CL > 8) cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)B * CL);
-    cfg.blockDim = dim3(CL == 9 ? 512 : soft_tile_threads(p));
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute at;
-    at.id = cudaLaunchAttributeClusterDimension;
-    at.val.clusterDim.x = CL;
-    at.val.clusterDim.y = at.val.clusterDim.z = 1;
-    cfg.attrs = &at;
-    cfg.numAttrs = CL > 1;
-    return cudaLaunchKernelEx(&cfg, kern, (const float *)c, p.nc, p.pair_base, (const float *)p.soft_d,
-                              p.pair_off0, (long)p.nc0, (const float *)p.soft_tw, p.P, P_per, (float *)grid,
-                              idx, euler, score, n_cand);
+    return launch_clusters(kern, B, CL, CL == 9 ? 512 : soft_tile_threads(p), smem, st, (const float *)c, p.nc,
+                           p.pair_base, (const float *)p.soft_d, p.pair_off0, p.nc0, (const float *)p.soft_tw,
+                           p.P, P_per, (float *)grid, idx, euler, score, n_cand);
   }
   {
     size_t smem = soft_chunk_smem(p, sizeof(T));
     if (smem <= 227 * 1024 - 1024) {
-      cudaFuncSetAttribute(k_soft_chunk<T, SOFT_KB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)smem);
-      k_soft_chunk<T, SOFT_KB><<<B, CHUNK_THREADS, smem, st>>>(
-          c, p.nc, p.L0, p.ns, p.pair_base, (const T *)p.soft_d, p.pair_off0, p.nc0,
-          (const T *)p.soft_tw, p.P, P_per, grid, idx, euler, score, n_cand);
-      return cudaGetLastError();
+      auto kern = k_soft_chunk<T, SOFT_KB>;
+      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      // CTAs per particle: passes of the longest one (and the short one ahead) times the
+      // waves; two CTAs on an SM take a third longer.  40 particles in FP64, 36 points
+      // per angle: 829 us on one CTA each, 337 on three.
+      const int passes = (p.ns + SOFT_KB - 1) / SOFT_KB, one = sizeof(T) == 8 || 2 * (smem + 1024) > 228 * 1024 ? 1 : 2;
+      int CL = 1;
+      double best = 1e30;
+      for (int q = 1; q <= std::min(8, passes); ++q) {
+        if (q > 1 && (passes + q - 1) / q * (q - 1) >= passes) continue;  // a CTA without slices
+        const long n = (long)B * q, waves = (n + one * p.sms - 1) / (one * p.sms);
+        const double t = waves * ((passes + q - 1) / q + (q > 1 ? 0.6 : 0.0)) * (n > p.sms && one > 1 ? 1.33 : 1.0);
+        if (t < 0.95 * best) { best = t; CL = q; }
+      }
+      return launch_clusters(kern, B, CL, CHUNK_THREADS, smem, st, c, p.nc, p.L0, p.ns, p.pair_base,
+                             (const T *)p.soft_d, p.pair_off0, p.nc0, (const T *)p.soft_tw, p.P, P_per, grid,
+                             idx, euler, score, n_cand, CL);
     }
   }
   // with a grid to write, through memory rather than slice by slice on one CTA
