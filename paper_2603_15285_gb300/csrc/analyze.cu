@@ -554,7 +554,7 @@ static AnalyzeShape analyze_shape(const Plan &p, long volumes) {
   G = G >= 8 ? 8 : G >= 4 ? 4 : G >= 2 ? 2 : 1;
   while (G > 1 && (p.S % G != 0 || analyze2_smem<T>(p, G) > 100 * 1024)) G >>= 1;
   // three CTAs on 164 KB, or two where the box is large
-  const bool cap = sizeof(T) == 4 && G == 1 && p.N >= 88 && cost(1) <= (p.N > 128 ? 82 : 54) * 1024;
+  const bool cap = sizeof(T) == 4 && G == 1 && p.N >= 88 && cost(1) <= 164 * 1024 / (p.N > 128 ? 2 : 3);
   return {G, cap ? 71 : -1};
 }
 
