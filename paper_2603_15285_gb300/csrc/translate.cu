@@ -49,70 +49,97 @@ __device__ __forceinline__ float add_rn(float a, float b) { return __fadd_rn(a, 
 // ---- volume pose ------------------------------------------------------------
 // out_b(x) = vol_b(R_b^T (x - c0) + c0 - s_b), trilinear, zero outside, one
 // thread per output voxel.  R (row-major [B][9]) and s ([B][3]) are nullable
-// (identity, zero).  Bound by the corner loads: a CTA takes a brick of 16 x 4 x 4
-// voxels, whose rotated corners share cache lines in all directions (a run of 256
-// along x does not), and all index arithmetic is 32-bit: corner indices are
-// clamped next to the box before the conversion (they are outside all the same),
-// the weights keep the unclamped coordinates.  The pose is converted once per CTA
-// (conversions from FP64 run at its rate).  96 volumes of 64^3 in FP32: rotated 652
-// -> 260 us, shifted 266 -> 240, of which the traffic is 30; the issue slots are 75%
-// busy (coordinates, eight guarded corners, weights).
+// (identity, zero).  A CTA takes a brick of 16 x 4 x 4 STEPS voxels, whose rotated
+// corners share cache lines in all directions (a run of 256 along x does not); a
+// thread takes STEPS of them along z, which spreads the block's indices, the pose (its
+// conversion from FP64 runs at that rate) and the rows' products over them.  All index
+// arithmetic is 32-bit: corner indices are clamped next to the box before the
+// conversion (they are outside all the same), the weights keep the unclamped
+// coordinates; one test replaces the eight guards where all corners are inside.  96
+// volumes of 64^3 in FP32: rotated 652 -> 170 us, shifted 266 -> 111 (one voxel per
+// thread 260 and 240; two 208 and 140; four 185 and 122), of which the traffic is 30;
+// then the issue of coordinates and weights.
 constexpr int POSE_X = 16, POSE_Y = 4, POSE_Z = 4;
-template <typename T>
+template <typename T, int STEPS>
 __global__ void __launch_bounds__(POSE_X * POSE_Y * POSE_Z)
-k_pose_volume(int N, int nbx, int nby, const float *__restrict__ vol, long vstride,
+k_pose_volume(int N, int nbx, const float *__restrict__ vol, long vstride,
               const double *__restrict__ R, const double *__restrict__ sh, float *__restrict__ out) {
-  const long b = blockIdx.y;
-  const int bz = blockIdx.x / (nbx * nby), br = blockIdx.x - bz * nbx * nby, by = br / nbx;
-  const int i = (br - by * nbx) * POSE_X + threadIdx.x % POSE_X;
+  const long b = blockIdx.z;
+  const int by = blockIdx.x / nbx;
+  const int i = (blockIdx.x - by * nbx) * POSE_X + threadIdx.x % POSE_X;
   const int j = by * POSE_Y + threadIdx.x / POSE_X % POSE_Y;
-  const int k = bz * POSE_Z + threadIdx.x / (POSE_X * POSE_Y);
+  const int kb = blockIdx.y * POSE_Z * STEPS + threadIdx.x / (POSE_X * POSE_Y);
   __shared__ T r[12];  // R, then s: converted once, conversions from FP64 run at its rate
   if (threadIdx.x < 9) r[threadIdx.x] = R ? (T)R[9 * b + threadIdx.x] : T(threadIdx.x % 4 == 0);
   else if (threadIdx.x < 12) r[threadIdx.x] = sh ? (T)sh[3 * b + threadIdx.x - 9] : T(0);
   __syncthreads();
-  if (i >= N || j >= N || k >= N) return;
+  if (i >= N || j >= N) return;
   const float *src = vol + b * vstride;
+  float *dst = out + b * (long)N * N * N + j * N + i;
   const T s0 = r[9], s1 = r[10], s2 = r[11];
   const T c0 = T(0.5) * (T)N;
-  const T x = (T)i - c0, y = (T)j - c0, z = (T)k - c0;
+  const T x = (T)i - c0, y = (T)j - c0;
   // column c of R dotted with (x, y, z), then + c0 - s, left to right
-  T px = add_rn(add_rn(add_rn(add_rn(mul_rn(r[0], x), mul_rn(r[3], y)), mul_rn(r[6], z)), c0), -s0);
-  T py = add_rn(add_rn(add_rn(add_rn(mul_rn(r[1], x), mul_rn(r[4], y)), mul_rn(r[7], z)), c0), -s1);
-  T pz = add_rn(add_rn(add_rn(add_rn(mul_rn(r[2], x), mul_rn(r[5], y)), mul_rn(r[8], z)), c0), -s2);
-  const T fx0 = floor(px), fy0 = floor(py), fz0 = floor(pz);
-  // -2 .. N + 1 (a NaN gives -2): past the box on either side with both corners
-  const T lo = T(-2), hi = (T)(N + 1);
-  const int i0 = (int)fmin(fmax(fx0, lo), hi), j0 = (int)fmin(fmax(fy0, lo), hi),
-            k0 = (int)fmin(fmax(fz0, lo), hi);
-  const T tx = add_rn(px, -fx0), ty = add_rn(py, -fy0), tz = add_rn(pz, -fz0);
-  float val[8];
+  const T xy0 = add_rn(mul_rn(r[0], x), mul_rn(r[3], y)), xy1 = add_rn(mul_rn(r[1], x), mul_rn(r[4], y)),
+          xy2 = add_rn(mul_rn(r[2], x), mul_rn(r[5], y));
+  const T r6 = r[6], r7 = r[7], r8 = r[8];
+  const int NN = N * N;
 #pragma unroll
-  for (int q = 0; q < 8; ++q) {
-    const int ii = i0 + (q & 1), jj = j0 + (q >> 1 & 1), kk = k0 + (q >> 2);
-    val[q] = 0.f;
-    if ((unsigned)ii < (unsigned)N && (unsigned)jj < (unsigned)N && (unsigned)kk < (unsigned)N)
-      val[q] = __ldg(src + (kk * N + jj) * N + ii);
-  }
-  T acc = 0;
+  for (int q = 0; q < STEPS; ++q) {
+    const int k = kb + q * POSE_Z;
+    if (k >= N) break;
+    const T z = (T)k - c0;
+    const T px = add_rn(add_rn(add_rn(xy0, mul_rn(r6, z)), c0), -s0);
+    const T py = add_rn(add_rn(add_rn(xy1, mul_rn(r7, z)), c0), -s1);
+    const T pz = add_rn(add_rn(add_rn(xy2, mul_rn(r8, z)), c0), -s2);
+    const T fx0 = floor(px), fy0 = floor(py), fz0 = floor(pz);
+    // -2 .. N + 1 (a NaN gives -2): past the box on either side with both corners
+    const T lo = T(-2), hi = (T)(N + 1);
+    const int i0 = (int)fmin(fmax(fx0, lo), hi), j0 = (int)fmin(fmax(fy0, lo), hi),
+              k0 = (int)fmin(fmax(fz0, lo), hi);
+    const T tx = add_rn(px, -fx0), ty = add_rn(py, -fy0), tz = add_rn(pz, -fz0);
+    float val[8];
+    const unsigned last = N - 1;
+    if ((unsigned)i0 < last && (unsigned)j0 < last && (unsigned)k0 < last) {  // all corners inside
+      const float *p0 = src + (k0 * N + j0) * N + i0, *p1 = p0 + N, *p2 = p0 + NN, *p3 = p1 + NN;
+      val[0] = __ldg(p0); val[1] = __ldg(p0 + 1);
+      val[2] = __ldg(p1); val[3] = __ldg(p1 + 1);
+      val[4] = __ldg(p2); val[5] = __ldg(p2 + 1);
+      val[6] = __ldg(p3); val[7] = __ldg(p3 + 1);
+    } else {
 #pragma unroll
-  for (int q = 0; q < 8; ++q) {
-    const int dx = q & 1, dy = q >> 1 & 1, dz = q >> 2;
-    const T w = mul_rn(mul_rn(dx ? tx : add_rn(T(1), -tx), dy ? ty : add_rn(T(1), -ty)),
-                       dz ? tz : add_rn(T(1), -tz));
-    acc = add_rn(acc, mul_rn(w, (T)val[q]));
+      for (int c = 0; c < 8; ++c) {
+        const int ii = i0 + (c & 1), jj = j0 + (c >> 1 & 1), kk = k0 + (c >> 2);
+        val[c] = 0.f;
+        if ((unsigned)ii < (unsigned)N && (unsigned)jj < (unsigned)N && (unsigned)kk < (unsigned)N)
+          val[c] = __ldg(src + (kk * N + jj) * N + ii);
+      }
+    }
+    const T ux = add_rn(T(1), -tx), uy = add_rn(T(1), -ty), uz = add_rn(T(1), -tz);
+    T acc = 0;
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+      const T w = mul_rn(mul_rn(c & 1 ? tx : ux, c >> 1 & 1 ? ty : uy), c >> 2 ? tz : uz);
+      acc = add_rn(acc, mul_rn(w, (T)val[c]));
+    }
+    dst[k * NN] = (float)acc;
   }
-  out[b * (long)N * N * N + (k * N + j) * N + i] = (float)acc;
 }
 
 cudaError_t launch_pose_volumes(int N, const float *vol, int B, long vol_stride, const double *R,
                                 const double *shift, bool fp64, float *out, cudaStream_t st) {
   if (B <= 0) return cudaSuccess;
   const int nbx = (N + POSE_X - 1) / POSE_X, nby = (N + POSE_Y - 1) / POSE_Y;
-  dim3 grid((unsigned)(nbx * nby * ((N + POSE_Z - 1) / POSE_Z)), B);
   constexpr int threads = POSE_X * POSE_Y * POSE_Z;
-  if (fp64) k_pose_volume<double><<<grid, threads, 0, st>>>(N, nbx, nby, vol, vol_stride, R, shift, out);
-  else k_pose_volume<float><<<grid, threads, 0, st>>>(N, nbx, nby, vol, vol_stride, R, shift, out);
+  auto run = [&](auto steps) {
+    constexpr int ST = decltype(steps)::value;
+    const dim3 grid((unsigned)(nbx * nby), (unsigned)((N + POSE_Z * ST - 1) / (POSE_Z * ST)), B);
+    if (fp64) k_pose_volume<double, ST><<<grid, threads, 0, st>>>(N, nbx, vol, vol_stride, R, shift, out);
+    else k_pose_volume<float, ST><<<grid, threads, 0, st>>>(N, nbx, vol, vol_stride, R, shift, out);
+  };
+  // eight voxels per thread where that still makes four CTAs on each of 152 SMs
+  if ((long)nbx * nby * ((N + 31) / 32) * B >= 608) run(std::integral_constant<int, 8>{});
+  else run(std::integral_constant<int, 2>{});
   return cudaGetLastError();
 }
 
