@@ -33,7 +33,7 @@
 namespace matcha {
 namespace {
 
-constexpr int BWD_THREADS = 256, POINT_THREADS = 128;
+constexpr int BWD_THREADS = 256;
 
 // first (group, l) entry of group (m, j) in the grouped layout:
 // sum_{m' < m} (m'+1)(L-m'+1) + j (L-m+1)
@@ -97,8 +97,8 @@ __device__ __forceinline__ void seed3(int m, int n, T K, const T *ch, const T *s
 __device__ __forceinline__ void add_img(double (&acc)[10], double W, double u, double v, double er,
                                         double ei, double s0r, double s0i, double s1r, double s1i,
                                         double s2r, double s2i) {
-  const double zr0 = s0r * er - s0i * ei, zi0 = s0r * ei + s0i * er;
-  const double zr1 = s1r * er - s1i * ei, zi1 = s1r * ei + s1i * er;
+  const double zr0 = s0r * er - s0i * ei, zi0 = __fma_rn(s0i, er, __dmul_rn(s0r, ei));
+  const double zr1 = s1r * er - s1i * ei, zi1 = __fma_rn(s1i, er, __dmul_rn(s1r, ei));
   const double zr2 = s2r * er - s2i * ei;
   acc[0] += W * zr0;
   acc[1] -= W * u * zi0;
@@ -172,31 +172,26 @@ __device__ __forceinline__ void load8(const T *p, T (&v)[8]) {
 //
 // A thread takes the two pairs (m, n) of a group along their l-recurrence, a record
 // of c and one of the coefficients per degree, the next ones in flight.  Bound by the
-// FP64 pipe: the sums of the images stay in FP64, their phases are products of the
-// particle's tables of cos and sin (k a), (k g) (a sincos per image and a shuffle tree
-// of FP64 additions were more than half of the work).  512 particles, L_J = 32, FP32:
-// 318 -> 127 us; CTAs of 128 threads, of which four fit an SM and one wave holds the
-// batch (256 threads: 141).
+// FP64 pipe (64 cycles of a quarter SM per warp and operation): a sincos and about
+// thirty operations per image.  At a refined rotation grad C is a cancelled sum whose
+// last bits carry over into v, so the phases, the order of the sums and the tree of the
+// reduction are part of the result; the tree is evaluated by all threads from shared
+// memory, not as 50 shuffled additions in every warp.  512 particles, L_J = 32, FP32:
+// 318 -> 198 us (the pipe alone: about 170).
 template <typename T, bool VEC>
-__global__ void __launch_bounds__(POINT_THREADS)
+__global__ void __launch_bounds__(BWD_THREADS)
     k_bwd_point(const T *__restrict__ c, long cper, const T *__restrict__ rcoef,
                 const T *__restrict__ seedK, int L, const double *__restrict__ euler,
                 double *__restrict__ shift, int *__restrict__ flags) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  double *red = reinterpret_cast<double *>(smem_raw);  // [10][POINT_THREADS + 1]
-  double2 *ta = reinterpret_cast<double2 *>(red + 10 * (POINT_THREADS + 1)), *tg = ta + L + 1;
-  T *chp = reinterpret_cast<T *>(tg + L + 1), *shp = chp + pw_len(L);
+  double *red = reinterpret_cast<double *>(smem_raw);  // [10][BWD_THREADS]
+  T *chp = reinterpret_cast<T *>(red + 10 * BWD_THREADS), *shp = chp + pw_len(L);
   const long b = blockIdx.x;
   const T *cb = c + b * cper;
   const double al = euler[3 * b], be = euler[3 * b + 1], ga = euler[3 * b + 2];
   T trig[4];
   beta_trig(be, trig);
   const T x = trig[0], s = trig[1], ch = trig[2], sh = trig[3];
-  for (int k = threadIdx.x; k < 2 * (L + 1); k += blockDim.x) {
-    double2 e;
-    sincos(k <= L ? k * al : (k - L - 1) * ga, &e.y, &e.x);
-    ta[k] = e;
-  }
   power_tables(chp, shp, pw_len(L), ch, sh);
   __syncthreads();
   double acc[10];
@@ -248,35 +243,35 @@ __global__ void __launch_bounds__(POINT_THREADS)
     for (int h = 0; h < 2; ++h) {
       const int n = 2 * j - m + h;
       if (n > m) break;
-      const double2 am = ta[m], gm = tg[m];
-      double2 an = ta[abs(n)], gn = tg[abs(n)];
-      if (n < 0) { an.y = -an.y; gn.y = -gn.y; }
+      double sn, cn;
       // image (m, n), weight 1 for (0, 0) else 2 (with its conjugate (-m, -n))
-      add_img(acc, (m == 0 && n == 0) ? 1.0 : 2.0, m, n, am.x * gn.x - am.y * gn.y,
-              am.y * gn.x + am.x * gn.y, s0r[h], s0i[h], s1r[h], s1i[h], s2r[h], s2i[h]);
+      sincos(m * al + n * ga, &sn, &cn);
+      add_img(acc, (m == 0 && n == 0) ? 1.0 : 2.0, m, n, cn, sn, s0r[h], s0i[h], s1r[h], s1i[h], s2r[h],
+              s2i[h]);
       // image (n, m): d^l_nm = (-1)^{m-n} d^l_mn; absent for n = +-m
-      if (n != m && n != -m)
-        add_img(acc, ((m - n) & 1) ? -2.0 : 2.0, n, m, an.x * gm.x - an.y * gm.y,
-                an.y * gm.x + an.x * gm.y, t0r[h], t0i[h], t1r[h], t1i[h], t2r[h], t2i[h]);
+      if (n != m && n != -m) {
+        sincos(n * al + m * ga, &sn, &cn);
+        add_img(acc, ((m - n) & 1) ? -2.0 : 2.0, n, m, cn, sn, t0r[h], t0i[h], t1r[h], t1i[h], t2r[h],
+                t2i[h]);
+      }
     }
   }
-  // the block's sums: a thread adds 32 terms of one quantity
+  // a warp's 32 terms as the tree (i, i + 16), (i, i + 8), ..., then the warps in order
 #pragma unroll
-  for (int i = 0; i < 10; ++i) red[i * (POINT_THREADS + 1) + threadIdx.x] = acc[i];
-  __syncthreads();
-  constexpr int SEG = POINT_THREADS / 32;
-  double part = 0.0;
-  const int iq = threadIdx.x / SEG, seg = threadIdx.x % SEG;
-  if (iq < 10)
-    for (int k = 0; k < 32; ++k) part += red[iq * (POINT_THREADS + 1) + seg + SEG * k];
-  __syncthreads();
-  if (iq < 10) red[threadIdx.x] = part;
+  for (int i = 0; i < 10; ++i) red[i * BWD_THREADS + threadIdx.x] = acc[i];
+  for (int o = 16; o > 0; o >>= 1) {
+    __syncthreads();
+    for (int t = threadIdx.x; t < 10 * (BWD_THREADS / 32) * o; t += BWD_THREADS) {
+      double *x = red + t / o * 32 + t % o;
+      x[0] += x[o];
+    }
+  }
   __syncthreads();
   if (threadIdx.x == 0) {
     double r[10];
     for (int i = 0; i < 10; ++i) {
       r[i] = 0.0;
-      for (int w = 0; w < SEG; ++w) r[i] += red[i * SEG + w];
+      for (int w = 0; w < BWD_THREADS / 32; ++w) r[i] += red[i * BWD_THREADS + 32 * w];
     }
     const double grad[3] = {r[1], r[2], r[3]};
     const double H[9] = {r[4], r[5], r[6], r[5], r[7], r[8], r[6], r[8], r[9]};
@@ -298,6 +293,10 @@ __host__ __device__ __forceinline__ long bwd_coef_reals(int L, int shells) {
   return 4L * (L + 1) * (L + 1) + 2L * (2 * L + 1) * bwd_cols(L) + 4L * (2 * L + 1) + 2L * pw_len(L) +
          2L * shells + 2 + 4L * shells * (L + 1);
 }
+
+// products that the compiler may not fuse
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
 
 // pairs of columns: packed in FP32
 __device__ __forceinline__ float2 p_mul(float a, float2 b) { return __fmul2_rn(make_float2(a, a), b); }
@@ -429,7 +428,7 @@ __global__ void __launch_bounds__(BWD_THREADS, sizeof(T) == 4 ? 4 : 2)
         const T ar = pa[2 * (u + L)], ai = pa[2 * (u + L) + 1];
         const T gr = pg[2 * (w + L)], gi = pg[2 * (w + L) + 1];
         const T er = ar * gr - ai * gi, ei = ar * gi + ai * gr;
-        const T br = dd - vb * dd1, bi = -(tu * va + tw * vg) * dd;
+        const T br = dd - vb * dd1, bi = -fma(tw, vg, mul_rn(tu, va)) * dd;
         T *o = Es + 2 * ((u + L) * LN + (w & ~1)) + (w & 1);
         o[0] = er * br - ei * bi;
         o[2] = er * bi + ei * br;
@@ -628,10 +627,9 @@ cudaError_t launch_template_grad(const Plan &p, const T *f, const T *c, int B, i
   if (B == 0) return cudaSuccess;
   const long per = 2L * p.S * p.nlm;
   const bool vec = (uintptr_t)c % 16 == 0;
-  const size_t ps = sizeof(double) * (10 * (POINT_THREADS + 1) + 4 * (size_t)(p.LJ + 1)) +
-                    2 * sizeof(T) * pw_len(p.LJ);
+  const size_t ps = sizeof(double) * 10 * BWD_THREADS + 2 * sizeof(T) * pw_len(p.LJ);
   auto point = vec ? k_bwd_point<T, true> : k_bwd_point<T, false>;
-  point<<<B, POINT_THREADS, ps, st>>>(c, 4L * p.nc, (const T *)p.rcoef, (const T *)p.seedK, p.LJ, euler,
+  point<<<B, BWD_THREADS, ps, st>>>(c, 4L * p.nc, (const T *)p.rcoef, (const T *)p.seedK, p.LJ, euler,
                                     shift, flags);
   // Shells per CTA: all of them where the batch fills the chip twice over, else split
   // (each CTA repeats the recurrence); fewer where the coefficients do not fit.
