@@ -583,8 +583,9 @@ cudaError_t launch_analyze(const Plan &p, const float *vols, int B, T *coef, cud
       // threads and 1.59 with 128)
       auto run = [&](bool x, const float *v, int n, T *o, int n2) {
         auto kern = x ? pick(std::true_type{}) : pick(std::false_type{});
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, sh.carve);
+        // the calls that a launch needs: small ones are bound by the host
+        if (smem > 44 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (G == 1) cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, sh.carve);
         kern<<<dim3(p.S / G, n + n2), ANALYZE_THREADS, smem, st>>>(
             v, n, vols2, p.N, p.S, p.LJ, p.rs, p.xj, (const T *)p.phi_cs, (const T *)p.dft_cs, p.Mp, p.Qf,
             p.Mq, (const T *)p.ptab_leg, p.leg_lm, (const T *)p.ring, o, coef2, tp);
