@@ -790,9 +790,13 @@ cudaError_t launch_shift_search(const Plan &p, const float *f, const float *u, i
     k_fft_plane<T><<<dim3(N, B), 256, plane, st>>>(Z, f, u, fd, tw);
   } else {
     // rows, then columns (at least 16, so their rows stay coalesced), about 4096
-    // elements per CTA
-    const int NB0 = 4096 / N > 0 ? 4096 / N : 1, NB = 4096 / N > 16 ? 4096 / N : 16;
-    const size_t sm0 = cs * (2 * (size_t)NB0 * (N | 1) + N), sm1 = cs * (2 * (size_t)NB * (N | 1) + N);
+    // elements per CTA; fewer where they and the twiddles exceed shared memory (FP64
+    // from N = 450 on: eight columns, 128 bytes of a row)
+    auto lines = [&](int nb) { return cs * (2 * (size_t)nb * (N | 1) + N); };
+    const int NB0 = 4096 / N > 0 ? 4096 / N : 1;
+    int NB = 4096 / N > 16 ? 4096 / N : 16;
+    while (lines(NB) > 227 * 1024) NB /= 2;
+    const size_t sm0 = lines(NB0), sm1 = lines(NB);
     cudaFuncSetAttribute(k_fft_axis<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)(sm0 > sm1 ? sm0 : sm1));
     k_fft_axis<T><<<dim3((unsigned)((N2 + NB0 - 1) / NB0), B), 256, sm0, st>>>(Z, f, u, 0, fd, tw, NB0);
