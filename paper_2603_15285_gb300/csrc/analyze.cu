@@ -558,6 +558,8 @@ static AnalyzeShape analyze_shape(const Plan &p, long volumes) {
   return {G, cap ? 71 : -1};
 }
 
+static std::mutex carve_mu;
+
 // Analyses B volumes into coef and, in the same launch where it can, B2 into coef2.
 template <typename T>
 cudaError_t launch_analyze(const Plan &p, const float *vols, int B, T *coef, cudaStream_t st,
@@ -583,9 +585,14 @@ cudaError_t launch_analyze(const Plan &p, const float *vols, int B, T *coef, cud
       // threads and 1.59 with 128)
       auto run = [&](bool x, const float *v, int n, T *o, int n2) {
         auto kern = x ? pick(std::true_type{}) : pick(std::false_type{});
-        // the calls that a launch needs: small ones are bound by the host
-        if (smem > 44 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (G == 1) cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, sh.carve);
+        const cudaError_t e = allow_smem(kern, smem);
+        if (e != cudaSuccess) return e;
+        // the carve-out, too, is one value per kernel: no other thread's between it and the launch
+        std::unique_lock<std::mutex> own(carve_mu, std::defer_lock);
+        if (G == 1) {
+          own.lock();
+          cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, sh.carve);
+        }
         kern<<<dim3(p.S / G, n + n2), ANALYZE_THREADS, smem, st>>>(
             v, n, vols2, p.N, p.S, p.LJ, p.rs, p.xj, (const T *)p.phi_cs, (const T *)p.dft_cs, p.Mp, p.Qf,
             p.Mq, (const T *)p.ptab_leg, p.leg_lm, (const T *)p.ring, o, coef2, tp);
@@ -608,7 +615,8 @@ cudaError_t launch_analyze(const Plan &p, const float *vols, int B, T *coef, cud
   while (RB > 1 && sizeof(T) * (fixed + (size_t)RB * p.np) > 220 * 1024) RB = (RB + 1) / 2;
   size_t smem = sizeof(T) * (fixed + (size_t)RB * p.np);
   if (smem > 220 * 1024) return cudaErrorInvalidConfiguration;
-  cudaFuncSetAttribute(k_analyze<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const cudaError_t e = allow_smem(k_analyze<T>, smem);
+  if (e != cudaSuccess) return e;
   k_analyze<T><<<dim3(p.S, B), 256, smem, st>>>(vols, p.N, p.S, p.LJ, p.rs, p.xj, (const T *)p.ptab,
                                                  (const T *)p.phi_cs, coef, RB);
   return cudaGetLastError();

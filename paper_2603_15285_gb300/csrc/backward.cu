@@ -629,33 +629,35 @@ cudaError_t launch_template_grad(const Plan &p, const T *f, const T *c, int B, i
   const bool vec = (uintptr_t)c % 16 == 0;
   const size_t ps = sizeof(double) * 10 * BWD_THREADS + 2 * sizeof(T) * pw_len(p.LJ);
   auto point = vec ? k_bwd_point<T, true> : k_bwd_point<T, false>;
-  point<<<B, BWD_THREADS, ps, st>>>(c, 4L * p.nc, (const T *)p.rcoef, (const T *)p.seedK, p.LJ, euler,
-                                    shift, flags);
   // Shells per CTA: all of them where the batch fills the chip twice over, else split
   // (each CTA repeats the recurrence); fewer where the coefficients do not fit.
   int parts = 1;
   while (2L * parts * BWD_TS <= p.S && (long)B * parts < 2L * p.sms) parts *= 2;
   int Sc = (p.S + parts - 1) / parts;
   Sc = (Sc + BWD_TS - 1) / BWD_TS * BWD_TS;
-  const size_t most = 227 * 1024 / sizeof(T);
+  const size_t most = SMEM_MOST / sizeof(T) - 4;
   while (Sc > 1 && (size_t)bwd_coef_reals(p.LJ, Sc) > most) --Sc;
   const size_t smem = sizeof(T) * (size_t)bwd_coef_reals(p.LJ, Sc);
-  cudaFuncSetAttribute(k_bwd_coef<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem(k_bwd_coef<T>, smem, 4 * sizeof(T));
+  if (e != cudaSuccess) return e;
   T *Xo = tstride ? coef_grad : X;
+  point<<<B, BWD_THREADS, ps, st>>>(c, 4L * p.nc, (const T *)p.rcoef, (const T *)p.seedK, p.LJ, euler,
+                                    shift, flags);
   k_bwd_coef<T><<<dim3(B, (p.S + Sc - 1) / Sc), BWD_THREADS, smem, st>>>(
       f, p.S, Sc, p.LJ, p.wrad, (const T *)p.rcoef, (const T *)p.seedK, euler, shift, weight, Xo);
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
   const int ntmpl = tstride ? B : 1;
   if (!tstride)
     k_bwd_reduce<T><<<(int)((per + RED_X - 1) / RED_X), dim3(RED_X, RED_Y), 0, st>>>(X, B, per, coef_grad);
   if (vox_grad) {
     const long nv = (long)p.N * p.N * p.N * ntmpl;
-    cudaError_t e = cudaMemsetAsync(vox_grad, 0, sizeof(double) * nv, st);
+    e = cudaMemsetAsync(vox_grad, 0, sizeof(double) * nv, st);
     if (e != cudaSuccess) return e;
     // rings per CTA: a shell's, or few enough that there are four CTAs per SM
     const int nt = p.LJ + 1, want = (int)(4L * p.sms / ((long)p.S * ntmpl) + 1);
     const int JB = (nt + want - 1) / want;
     const size_t ss = sizeof(T) * (2 * (size_t)JB * nt + 2 * (size_t)(2 * p.LJ + 2));
-    cudaFuncSetAttribute(k_bwd_synth<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ss);
+    if ((e = allow_smem(k_bwd_synth<T>, ss)) != cudaSuccess) return e;
     k_bwd_synth<T><<<dim3(p.S, ntmpl, (nt + JB - 1) / JB), BWD_THREADS, ss, st>>>(
         coef_grad, p.S, p.LJ, p.N, JB, (const T *)p.ptab, (const T *)p.phi_cs, (const T *)p.ring, vox_grad);
   }

@@ -290,8 +290,8 @@ cudaError_t launch_correlate(const Plan &p, const T *f, const T *h, int B, int h
   const size_t smem = out ? both : stage;
   auto kern = ball ? (out ? k_correlate_deg<T, true, true> : k_correlate_deg<T, true, false>)
                    : (out ? k_correlate_deg<T, false, true> : k_correlate_deg<T, false, false>);
-  if (smem > 44 * 1024)  // beyond what a launch may have unasked (48 KB with the static part)
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const cudaError_t e = allow_smem(kern, smem, 256 * sizeof(T));
+  if (e != cudaSuccess) return e;
   kern<<<dim3(p.LJ / 2 + 1, B), threads, smem, st>>>(f, h, p.S, p.LJ, hstride, p.wrad, p.pair_base, p.nc, c,
                                                      ball ? (const T *)p.ball_W : nullptr,
                                                      ball ? p.ball_K : nullptr, ball ? p.ball_kmax : 0);

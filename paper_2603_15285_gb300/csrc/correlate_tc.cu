@@ -724,7 +724,8 @@ cudaError_t launch_correlate_tc(const Plan &p, const float *f, const float *h, i
     const int smem1 = (int)tc_shared(g, p.LJ, PM).smem;
     const long limit = p.wait_limit >= 0 ? p.wait_limit : TC_WAIT_LIMIT;
     auto kern = bf16 ? k_correlate_tc_shared<1> : k_correlate_tc_shared<0>;
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem1);
+    const cudaError_t e = allow_smem(kern, smem1, 1024);
+    if (e != cudaSuccess) return e;
     kern<<<(int)(units < nsm ? units : nsm), TS_THREADS, smem1, st>>>(f, h, p.S, p.LJ, p.wrad, p.nc, c, B,
                                                                       PB, PM, p.dev_err, limit);
     return cudaGetLastError();
@@ -734,12 +735,12 @@ cudaError_t launch_correlate_tc(const Plan &p, const float *f, const float *h, i
   const int grid = (int)(items < per_sm * nsm ? items : per_sm * nsm);
   const size_t smem = (size_t)tc_smem(g);
   const long wait_limit = p.wait_limit >= 0 ? p.wait_limit : TC_WAIT_LIMIT;
+  const cudaError_t e = bf16 ? allow_smem(k_correlate_tc<1>, smem, 1024) : allow_smem(k_correlate_tc<0>, smem, 1024);
+  if (e != cudaSuccess) return e;
   if (bf16) {
-    cudaFuncSetAttribute(k_correlate_tc<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     k_correlate_tc<1><<<grid, TC_THREADS, smem, st>>>(f, h, p.S, p.LJ, hstride, p.wrad, p.nc, c, B,
                                                       p.dev_err, wait_limit);
   } else {
-    cudaFuncSetAttribute(k_correlate_tc<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     k_correlate_tc<0><<<grid, TC_THREADS, smem, st>>>(f, h, p.S, p.LJ, hstride, p.wrad, p.nc, c, B,
                                                       p.dev_err, wait_limit);
   }

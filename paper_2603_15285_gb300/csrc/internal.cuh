@@ -103,6 +103,21 @@ void destroy_texsets(Plan &p);
 
 inline size_t align_up(size_t x, size_t a = 256) { return (x + a - 1) / a * a; }
 
+// Opts a kernel in to a launch with `bytes` of dynamic shared memory; `fixed` is the
+// kernel's static part.  The limit is one value per kernel and device, shared by every
+// plan and host thread, so it is only ever set to the same value, the most that fits
+// beside the static part: a limit of each launch's own size could be lowered by another
+// thread between the call and the launch, which then fails.  Small launches need none.
+// More than fits is refused here, before the launch: where another launch follows, the
+// error of a failed one is not what cudaGetLastError returns.
+constexpr size_t SMEM_MOST = 227 * 1024;
+template <typename... Args>
+cudaError_t allow_smem(void (*kern)(Args...), size_t bytes, size_t fixed = 0) {
+  if (bytes <= 44 * 1024) return cudaSuccess;  // 48 KB with the static part
+  if (bytes + fixed > SMEM_MOST) return cudaErrorInvalidConfiguration;
+  return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(SMEM_MOST - fixed));
+}
+
 // Grouped correlation layout.  The order pairs (m, n), m >= |n|, of one m are
 // taken two at a time: group g = m(m+1)/2 + j (j = 0..m) holds the partners
 // n_a = 2j - m and n_b = n_a + 1 (half 0 and half 1); for j = m the second

@@ -850,13 +850,13 @@ cudaError_t launch_newton(const Plan &p, const T *c, int B, const int *n_cand, d
   size_t smem = newton_smem_bytes(p, sizeof(T), A.nslots);
   if constexpr (sizeof(T) == 4) {
     if (newton_rescaled(p)) {
-      cudaFuncSetAttribute(k_newton<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      if ((e = allow_smem(k_newton<T, true>, smem)) != cudaSuccess) return e;
       k_newton<T, true><<<B, NEWTON_THREADS, smem, st>>>(c, (const T *)p.rcoef, (const T *)p.seedK,
                                                          A, n_cand, euler, score, cflags, work);
       return cudaGetLastError();
     }
   }
-  cudaFuncSetAttribute(k_newton<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if ((e = allow_smem(k_newton<T, false>, smem)) != cudaSuccess) return e;
   k_newton<T, false><<<B, NEWTON_THREADS, smem, st>>>(c, (const T *)p.rcoef, (const T *)p.seedK,
                                                       A, n_cand, euler, score, cflags, work);
   return cudaGetLastError();
@@ -880,17 +880,18 @@ cudaError_t launch_newton_queue(const Plan &p, const T *c, int B, const int *n_c
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   auto go = [&](auto kern) {
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t e = allow_smem(kern, smem, 16);
+    if (e != cudaSuccess) return e;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, NEWTON_THREADS, smem);
     const int grid = std::max(1, std::min(B, std::max(per_sm, 1) * sms));
     kern<<<grid, NEWTON_THREADS, smem, st>>>(c, (const T *)p.rcoef, (const T *)p.seedK, A, n_cand,
                                              euler, score, cflags, work, order, B, ticket);
+    return cudaGetLastError();
   };
   if constexpr (sizeof(T) == 4) {
-    if (newton_rescaled(p)) { go(k_newton_queue<T, true>); return cudaGetLastError(); }
+    if (newton_rescaled(p)) return go(k_newton_queue<T, true>);
   }
-  go(k_newton_queue<T, false>);
-  return cudaGetLastError();
+  return go(k_newton_queue<T, false>);
 }
 template cudaError_t launch_newton_queue<float>(const Plan &, const float *, int, const int *,
                                                 double *, double *, int *, long long *, int *,
@@ -915,13 +916,13 @@ cudaError_t launch_objective(const Plan &p, const T *c, int B, int L, int Q, con
   size_t smem = newton_smem_bytes(p, sizeof(T), A.nslots);
   if constexpr (sizeof(T) == 4) {
     if (newton_rescaled(p)) {
-      cudaFuncSetAttribute(k_objective<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      if ((e = allow_smem(k_objective<T, true>, smem)) != cudaSuccess) return e;
       k_objective<T, true><<<B, NEWTON_THREADS, smem, st>>>(c, (const T *)p.rcoef,
                                                             (const T *)p.seedK, A, L, Q, pts, out);
       return cudaGetLastError();
     }
   }
-  cudaFuncSetAttribute(k_objective<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if ((e = allow_smem(k_objective<T, false>, smem)) != cudaSuccess) return e;
   k_objective<T, false><<<B, NEWTON_THREADS, smem, st>>>(c, (const T *)p.rcoef, (const T *)p.seedK,
                                                          A, L, Q, pts, out);
   return cudaGetLastError();

@@ -864,10 +864,8 @@ bool spread_shape(const Plan &p, size_t tsize, int B, SpreadArgs &out, size_t *s
 template <typename... Args>
 cudaError_t launch_clusters(void (*kern)(Args...), int B, const SpreadArgs &A, size_t smem,
                             cudaStream_t st, Args... args) {
-  if (smem > 44 * 1024) {
-    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-  }
+  const cudaError_t e = allow_smem(kern, smem);
+  if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeClusterDimension;

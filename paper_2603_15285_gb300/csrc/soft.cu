@@ -1263,7 +1263,8 @@ cudaError_t launch_soft(const Plan &p, const T *c, int B, const int *P_per, T *g
   // for 256 particles)
   if (sizeof(T) == 4 && p.tune_soft == 2 && soft_warps_ok(p)) {
     size_t smem = soft_warps_smem<SOFT_NW>(p);
-    cudaFuncSetAttribute(k_soft_warps<SOFT_NW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t e = allow_smem(k_soft_warps<SOFT_NW>, smem);
+    if (e != cudaSuccess) return e;
     k_soft_warps<SOFT_NW><<<B, SOFT_NW * 32, smem, st>>>(
         (const float *)c, p.nc, p.L0, p.ns, p.pair_base, (const float *)p.soft_d, p.pair_off0,
         p.nc0, (const float *)p.soft_tw, p.P, P_per, (float *)grid, idx, euler, score, n_cand);
@@ -1277,7 +1278,8 @@ cudaError_t launch_soft(const Plan &p, const T *c, int B, const int *P_per, T *g
     const size_t smem = soft_tile_smem(p, CL > 1);
     auto kern = CL == 9 ? k_soft_split<TILE_KB, 8, 36, SOFT_SPLIT_MOST>
               : CL == 3 ? k_soft_split<TILE_KB, 8, 36, 3> : k_soft_tile<TILE_KB, 8, 36>;
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t e = allow_smem(kern, smem);
+    if (e != cudaSuccess) return e;
     return launch_clusters(kern, B, CL, CL == 9 ? 512 : soft_tile_threads(p), smem, st, (const float *)c, p.nc,
                            p.pair_base, (const float *)p.soft_d, p.pair_off0, p.nc0, (const float *)p.soft_tw,
                            p.P, P_per, (float *)grid, idx, euler, score, n_cand);
@@ -1286,7 +1288,8 @@ cudaError_t launch_soft(const Plan &p, const T *c, int B, const int *P_per, T *g
     size_t smem = soft_chunk_smem(p, sizeof(T));
     if (smem <= 227 * 1024 - 1024) {
       auto kern = k_soft_chunk<T, SOFT_KB>;
-      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      const cudaError_t e = allow_smem(kern, smem);
+      if (e != cudaSuccess) return e;
       // CTAs per particle: passes of the longest one (and the short one ahead) times the
       // waves; two CTAs on an SM take a third longer.  40 particles in FP64, 36 points
       // per angle: 829 us on one CTA each, 337 on three.
@@ -1309,7 +1312,8 @@ cudaError_t launch_soft(const Plan &p, const T *c, int B, const int *P_per, T *g
   const size_t smem = soft_stream_smem(p, sizeof(T));
   if (grid || smem > 227 * 1024 - 1024)
     return launch_soft_grid<T>(p, c, B, P_per, grid, idx, euler, score, n_cand, st);
-  cudaFuncSetAttribute(k_soft_stream<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const cudaError_t e = allow_smem(k_soft_stream<T>, smem);
+  if (e != cudaSuccess) return e;
   k_soft_stream<T><<<B, STREAM_THREADS, smem, st>>>(
       c, p.nc, p.L0, p.ns, p.pair_base, (const T *)p.soft_d, p.pair_off0, p.nc0,
       (const T *)p.soft_tw, p.P, P_per, grid, idx, euler, score, n_cand);

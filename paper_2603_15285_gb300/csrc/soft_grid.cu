@@ -702,9 +702,6 @@ cudaError_t launch_soft_grid(const Plan &p, const T *c, int B, const int *P_per,
   const int ng = (p.L0 + 1) * (p.L0 + 2) / 2;
   const bool vec = p.ns % 4 == 0 && reinterpret_cast<uintptr_t>(grid) % 16 == 0;
   const bool cvec = vec && reinterpret_cast<uintptr_t>(c) % 16 == 0;
-  (cvec ? k_soft_beta<T, true> : k_soft_beta<T, false>)
-      <<<dim3((ng + BETA_GROUPS - 1) / BETA_GROUPS, (B + BETA_NB - 1) / BETA_NB), 128, 0, st>>>(
-          c, p.nc, p.LJ, p.L0, p.ns, B, (const T *)p.soft_dT, grid);
   // beta slices per CTA: as many as give its threads one tile each, while the
   // batch still fills two CTAs on every SM and two fit an SM
   const int tiles = (round_up(p.ns, Tile<T>::I) / Tile<T>::I) * (round_up(p.ns, Tile<T>::J) / Tile<T>::J);
@@ -713,9 +710,15 @@ cudaError_t launch_soft_grid(const Plan &p, const T *c, int B, const int *P_per,
   const int IC = (int)slab_rows<T>(p, KS);
   if (IC == 0) return cudaErrorInvalidConfiguration;
   const size_t smem = sizeof(T) * slab_reals<T>(p.L0, p.ns, KS, IC);
-  cudaFuncSetAttribute(k_soft_slab<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem(k_soft_slab<T>, smem);
+  if (e != cudaSuccess) return e;
+  (cvec ? k_soft_beta<T, true> : k_soft_beta<T, false>)
+      <<<dim3((ng + BETA_GROUPS - 1) / BETA_GROUPS, (B + BETA_NB - 1) / BETA_NB), 128, 0, st>>>(
+          c, p.nc, p.LJ, p.L0, p.ns, B, (const T *)p.soft_dT, grid);
   k_soft_slab<T><<<dim3((p.ns + KS - 1) / KS, B), 256, smem, st>>>(p.L0, p.ns, KS, IC,
                                                                    (const T *)p.soft_tw, grid, vec);
+  e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
   // CTAs per particle: as many as the SMs take at two each
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute at[1];

@@ -750,17 +750,18 @@ static cudaError_t idft_grid(const Plan &p, int B, int nt, const double *org, in
   // the y stage are short, one column keeps their CTAs many (11 points: 23 against 33 us)
   auto midz = pick(std::integral_constant<int, 2>{}), midy = pick(std::integral_constant<int, 1>{});
   const size_t smem = 2 * cs * (size_t)N * JB;
-  cudaFuncSetAttribute(midz, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  cudaFuncSetAttribute(midy, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  // x stage: Y2[b][tz ty][kx] -> CC[b][tz ty][tx]
+  const int rows = nt * nt;
+  const size_t smx = cs * (8 * (size_t)N + (size_t)N * nt);
+  cudaError_t e;
+  if ((e = allow_smem(midz, smem)) != cudaSuccess || (e = allow_smem(midy, smem)) != cudaSuccess ||
+      (e = allow_smem(k_idft_x<T>, smx)) != cudaSuccess)
+    return e;
   const int ty = N <= 64 ? 64 : 128;
   midz<<<dim3((unsigned)((N2 + 255) / 256), 1, B), 128, smem, st>>>(
       (const C2<T> *)w.Z, (C2<T> *)w.Y1, (const C2<T> *)w.E, N, nt, 1, (int)N2, 2, es);
   midy<<<dim3((N + ty - 1) / ty, nt, B), ty, smem, st>>>(
       (const C2<T> *)w.Y1, (C2<T> *)w.Y2, (const C2<T> *)w.E, N, nt, nt, N, 1, es);
-  // x stage: Y2[b][tz ty][kx] -> CC[b][tz ty][tx]
-  const int rows = nt * nt;
-  size_t smx = cs * (8 * (size_t)N + (size_t)N * nt);
-  cudaFuncSetAttribute(k_idft_x<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smx);
   k_idft_x<T><<<dim3((rows + 7) / 8, B), 256, smx, st>>>(
       (const C2<T> *)w.Y2, (T *)w.CC, (const C2<T> *)w.E, N, nt, rows, T(1.0 / ((double)N2 * N)), es);
   k_cc_argmax<T><<<B, 256, 0, st>>>((const T *)w.CC, nt, org, j0, den, edge, flag_mode, R, t_out,
@@ -784,9 +785,10 @@ cudaError_t launch_shift_search(const Plan &p, const float *f, const float *u, i
   const C2<T> *tw = (const C2<T> *)p.fft_tw;
   // planes of which two buffers fit an SM (N <= 112 in FP32, 79 in FP64) are transformed
   // whole; larger ones a direction at a time
+  cudaError_t e;
   const size_t plane = cs * (2 * (size_t)N * (N | 1) + N);
   if (plane <= 200 * 1024) {
-    cudaFuncSetAttribute(k_fft_plane<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)plane);
+    if ((e = allow_smem(k_fft_plane<T>, plane)) != cudaSuccess) return e;
     k_fft_plane<T><<<dim3(N, B), 256, plane, st>>>(Z, f, u, fd, tw);
   } else {
     // rows, then columns (at least 16, so their rows stay coalesced), about 4096
@@ -795,10 +797,9 @@ cudaError_t launch_shift_search(const Plan &p, const float *f, const float *u, i
     auto lines = [&](int nb) { return cs * (2 * (size_t)nb * (N | 1) + N); };
     const int NB0 = 4096 / N > 0 ? 4096 / N : 1;
     int NB = 4096 / N > 16 ? 4096 / N : 16;
-    while (lines(NB) > 227 * 1024) NB /= 2;
+    while (lines(NB) > SMEM_MOST) NB /= 2;
     const size_t sm0 = lines(NB0), sm1 = lines(NB);
-    cudaFuncSetAttribute(k_fft_axis<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)(sm0 > sm1 ? sm0 : sm1));
+    if ((e = allow_smem(k_fft_axis<T>, sm0 > sm1 ? sm0 : sm1)) != cudaSuccess) return e;
     k_fft_axis<T><<<dim3((unsigned)((N2 + NB0 - 1) / NB0), B), 256, sm0, st>>>(Z, f, u, 0, fd, tw, NB0);
     k_fft_axis<T><<<dim3((unsigned)(N * ((N + NB - 1) / NB)), B), 256, sm1, st>>>(Z, nullptr, nullptr, 1,
                                                                                fd, tw, NB);
@@ -808,11 +809,11 @@ cudaError_t launch_shift_search(const Plan &p, const float *f, const float *u, i
   int NBz = 128 / (int)cs;
   while (NBz > 1 && cs * (4 * (size_t)NBz + 1) * N > 112 * 1024) NBz /= 2;
   const size_t smz = cs * (4 * (size_t)NBz + 1) * N;
-  cudaFuncSetAttribute(k_fft_cross<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smz);
+  if ((e = allow_smem(k_fft_cross<T>, smz)) != cudaSuccess) return e;
   const int nself = N % 2 ? 1 : 2, npair = (N - nself) / 2;
   const unsigned zt = nself * ((N / 2 + NBz) / NBz) + npair * ((N + NBz - 1) / NBz);
   k_fft_cross<T><<<dim3(zt, B), 128, smz, st>>>(Z, fd, tw, NBz);
-  cudaError_t e;
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
   // integer window [-m, m]^3
   const int nw = 2 * max_shift + 1;
   e = idft_grid<T>(p, B, nw, nullptr, -max_shift, 1, max_shift, 1, nullptr, w, w.t0,
