@@ -503,11 +503,21 @@ __global__ void __launch_bounds__(BWD_THREADS, sizeof(T) == 4 ? 4 : 2)
 
 // G[s][lm] = sum_b X[b][s][lm] (FP64 sums, fixed order).  A CTA takes RED_X elements
 // and RED_Y interleaved runs of b, RED_K particles at a time.  FP32: these are summed
-// as an FP32 value and the FP32 sum of its rounding errors (two-sum; what is lost is
-// below 2^-43 of the terms), which then enter the FP64 sum: FP64 conversions and
-// additions, which bound the plain loop, are an eighth.  512 x 35,904 values: 83 -> 19
-// us (reading them: 11).
+// as an unevaluated sum of three FP32 values (Knuth's two-sum: v enters s, the exact
+// rounding error of that enters e, and that one's enters r), which then enter the FP64
+// sum.  Only the additions into r round: with M the sum of the block's magnitudes, e is
+// below 15 2^-24 M and r below 120 2^-48 M, so less than 2^-61 M is lost, where FP64
+// additions of the 16 lose up to 15 2^-53 M.  FP64 conversions and additions, which
+// bound the plain loop, are three sixteenths.  512 x 35,904 values: 83 us as FP64
+// additions, 24 here (reading them: 11).
 constexpr int RED_X = 32, RED_Y = 8, RED_K = 16;
+// s + v into s; returns its rounding error, exact
+__device__ __forceinline__ float two_sum(float &s, float v) {
+  const float t = __fadd_rn(s, v), z = __fadd_rn(t, -s);
+  const float err = __fadd_rn(__fadd_rn(s, -__fadd_rn(t, -z)), __fadd_rn(v, -z));
+  s = t;
+  return err;
+}
 template <typename T>
 __global__ void __launch_bounds__(RED_X *RED_Y)
     k_bwd_reduce(const T *__restrict__ X, int B, long per, T *__restrict__ G) {
@@ -520,16 +530,13 @@ __global__ void __launch_bounds__(RED_X *RED_Y)
 #pragma unroll
       for (int k = 0; k < RED_K; ++k) v[k] = b0 + k < B ? X[(long)(b0 + k) * per + i] : T(0);
       if constexpr (sizeof(T) == 4) {
-        float s = v[0], e = 0.f;
+        float s = v[0], e = 0.f, r = 0.f;
 #pragma unroll
-        for (int k = 1; k < RED_K; ++k) {
-          const float t = __fadd_rn(s, v[k]), z = __fadd_rn(t, -s);
-          e = __fadd_rn(e, __fadd_rn(__fadd_rn(s, -__fadd_rn(t, -z)), __fadd_rn(v[k], -z)));
-          s = t;
-        }
+        for (int k = 1; k < RED_K; ++k) r = __fadd_rn(r, two_sum(e, two_sum(s, v[k])));
         if (isfinite(s)) {
           acc += (double)s;
           acc += (double)e;
+          acc += (double)r;
           continue;
         }
       }
