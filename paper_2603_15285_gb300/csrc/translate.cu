@@ -22,6 +22,7 @@
 // A pose kernel makes the rotated template u(x) = h(R^T (x - c0) + c0) and
 // the shifted template (S_tau h)(x) = h(x - tau) by trilinear interpolation.
 #include <math.h>
+#include <algorithm>
 #include <type_traits>
 #include "internal.cuh"
 
@@ -283,7 +284,7 @@ __device__ __forceinline__ void fft_lines(C2<T> *&src, C2<T> *&dst, const FftDes
   for (int q = 0; q < fd.npass; ++q) {
     int R = fd.radix[q];
     const bool head = q == 0;
-    if (R == 4 && q + 1 < fd.npass && fd.radix[q + 1] == 4) {
+    if (R == 4 && q + 1 < fd.npass && fd.radix[q + 1] == 4 && (sizeof(T) == 4 || NB * (N / 16) >= 32)) {
       R = 16;
       ++q;
     }
@@ -530,31 +531,45 @@ template <> struct CPair<float> { typedef float2 type; typedef float4 quad; };
 template <> struct CPair<double> { typedef double2 type; typedef Double4 quad; };
 
 // out[b][a][j][c] = sum_k in[b][a][k][c] E[b][axis][k][j]: the partial inverse
-// DFT along a middle (y) or outer (z) axis.  A thread takes CB columns c, JB grid
-// points j at a time in registers against the factors in shared memory (one 16-byte
-// broadcast per CB products of three packed operations); four rows k of its columns
-// are in flight while the four before are multiplied.  es: elements between the
-// particles' factors (0: shared).  96 volumes of 64^3 in FP32, 11 and 29 grid points:
-// the z stage 139 and 171 us -> 76 and 97 (one column per thread 97 and 117; two
-// without the loads ahead 128 and 143), then bound by its FMAs (floor 33) and, past
-// 16 points, by reading the volume again.
+// DFT along a middle (y) or outer (z) axis.  A thread takes CB of the A C columns (a, c)
+// of a particle, JB grid points j at a time in registers against the factors in shared
+// memory (one 16-byte broadcast per CB products of three packed operations); four rows
+// k of its columns are in flight while the four before are multiplied.  SP CTAs share a
+// tile of columns, each with every SP-th group of JB points.  es: elements between the
+// particles' factors (0: shared).
+//
+// FP32, SP = 1: 96 volumes of 64^3, 11 and 29 grid points: the z stage 139 and 171 us
+// -> 76 and 97 (one column per thread 97 and 117; two without the loads ahead 128 and
+// 143), then bound by its FMAs (floor 33) and, past 16 points, by reading the volume
+// again.  One volume, 41 points: 41 and 40 us in the z and y stages on 16 and 41 CTAs;
+// with one column and four points per CTA 14 and 12.
+// FP64: bound by its pipe, where an operation takes as long for one lane as for 32 and
+// a padded point as long as a real one, so no point is padded and the columns of all a
+// are packed into warps; one column, four points and a CTA per group of points spread the
+// work evenly.  64 volumes of 64^3, 41 points: 7.5 and 4.8 ms (eight padded points, two
+// columns in the z stage: 9.0 and 5.8); one volume: 165 and 112 us (1,304 and 633).
 template <typename T, int JB, int CB>
 __global__ void __launch_bounds__(128)
 k_idft_mid(const C2<T> *__restrict__ in, C2<T> *__restrict__ out, const C2<T> *__restrict__ E,
-           int N, int nt, int A, int C, int axis, long es) {
+           int N, int nt, int A, int C, int axis, long es, int SP) {
   typedef typename CPair<T>::type P2;
   typedef typename CPair<T>::quad Q;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   Q *Es = reinterpret_cast<Q *>(smem_raw);  // [N][JB]
   const long b = blockIdx.z;
-  const int a = blockIdx.y, c = blockIdx.x * blockDim.x * CB + threadIdx.x, tid = threadIdx.x;
-  const P2 *src = reinterpret_cast<const P2 *>(in) + (b * A + a) * (long)N * C + c;
-  const C2<T> *eb = E + b * es + (long)axis * N * nt;
-  P2 *dst = reinterpret_cast<P2 *>(out) + (b * A + a) * (long)nt * C + c;
-  int off[CB];  // a column past the end reads the thread's first
+  const int tile = blockIdx.x / SP, tid = threadIdx.x, cols = A * C;
+  const P2 *src[CB];
+  P2 *dst[CB];
+  const int c0 = tile * blockDim.x * CB + tid;
 #pragma unroll
-  for (int u = 0; u < CB; ++u) off[u] = c + u * (int)blockDim.x < C ? u * blockDim.x : 0;
-  for (int j0 = 0; j0 < nt; j0 += JB) {
+  for (int u = 0; u < CB; ++u) {  // a column past the end reads the thread's first
+    const int q = c0 + u * (int)blockDim.x < cols ? c0 + u * blockDim.x : min(c0, cols - 1);
+    const int a = q / C, c = q - a * C;
+    src[u] = reinterpret_cast<const P2 *>(in) + (b * A + a) * (long)N * C + c;
+    dst[u] = reinterpret_cast<P2 *>(out) + (b * A + a) * (long)nt * C + c;
+  }
+  const C2<T> *eb = E + b * es + (long)axis * N * nt;
+  for (int j0 = (blockIdx.x - tile * SP) * JB; j0 < nt; j0 += SP * JB) {
     __syncthreads();
     for (int t = tid; t < N * JB; t += blockDim.x) {
       const int k = t / JB, j = j0 + t % JB;
@@ -562,7 +577,8 @@ k_idft_mid(const C2<T> *__restrict__ in, C2<T> *__restrict__ out, const C2<T> *_
       Es[t] = Q{e.x, e.x, -e.y, e.y};
     }
     __syncthreads();
-    if (c >= C) continue;
+    if (c0 >= cols) continue;
+    const int nj = min(JB, nt - j0);
     P2 acc[CB][JB];
 #pragma unroll
     for (int u = 0; u < CB; ++u)
@@ -575,7 +591,7 @@ k_idft_mid(const C2<T> *__restrict__ in, C2<T> *__restrict__ out, const C2<T> *_
       for (int q = 0; q < U; ++q)
 #pragma unroll
         for (int u = 0; u < CB; ++u)
-          if (k0 + q < N) nx[q][u] = src[(long)(k0 + q) * C + off[u]];
+          if (k0 + q < N) nx[q][u] = src[u][(long)(k0 + q) * C];
     };
     load(0);
     for (int k0 = 0; k0 < N; k0 += U) {
@@ -590,6 +606,7 @@ k_idft_mid(const C2<T> *__restrict__ in, C2<T> *__restrict__ out, const C2<T> *_
         if (k0 + q >= N) break;
 #pragma unroll
         for (int j = 0; j < JB; ++j) {
+          if (sizeof(T) == 8 && j >= nj) break;
           const Q e = Es[(k0 + q) * JB + j];
 #pragma unroll
           for (int u = 0; u < CB; ++u) acc[u][j] = cmac(acc[u][j], v[q][u], e);
@@ -598,10 +615,10 @@ k_idft_mid(const C2<T> *__restrict__ in, C2<T> *__restrict__ out, const C2<T> *_
     }
 #pragma unroll
     for (int u = 0; u < CB; ++u)
-      if (u == 0 || off[u])
+      if (u == 0 || c0 + u * (int)blockDim.x < cols)
 #pragma unroll
         for (int j = 0; j < JB; ++j)
-          if (j0 + j < nt) dst[(long)(j0 + j) * C + off[u]] = acc[u][j];
+          if (j < nj) dst[u][(long)(j0 + j) * C] = acc[u][j];
   }
 }
 
@@ -735,33 +752,44 @@ static cudaError_t idft_grid(const Plan &p, int B, int nt, const double *org, in
   const long es = org ? 3L * N * nt : 0;
   k_idft_factors<T><<<3 * nb * ((N * nt + 255) / 256), 256, 0, st>>>((C2<T> *)w.E, N, nt, org, j0, den);
   // z stage: X[b][kz][ky kx] -> Y1[b][tz][ky kx], then y stage: Y1[b][tz][ky][kx]
-  // -> Y2[b][tz][ty][kx]; the grid points per pass over a column: the fewest passes
-  // of at most 16 (8 in FP64), rounded up to 4
+  // -> Y2[b][tz][ty][kx].  FP32: the grid points per pass over a column are the fewest
+  // passes of at most 16, rounded up to 4, with two columns per thread in the z stage,
+  // which has N^2 of them per volume (rows of the y stage are short, one column keeps
+  // their CTAs many: 11 points 23 against 33 us); where that makes fewer CTAs than SMs,
+  // and in FP64, one column and four points per CTA.
   const size_t cs = sizeof(C2<T>);
-  const int most = sizeof(T) == 8 ? 8 : 16, passes = (nt + most - 1) / most;
-  const int JB = ((nt + passes - 1) / passes + 3) / 4 * 4;
-  auto pick = [&](auto cb) {
+  const int passes = (nt + 15) / 16, wide = ((nt + passes - 1) / passes + 3) / 4 * 4;
+  const int narrow = (nt + 3) / 4, ty = N <= 64 ? 64 : 128;
+  const bool fewz = sizeof(T) == 8 || (N2 + 255) / 256 * B < p.sms;
+  const bool fewy = sizeof(T) == 8 || (long)((N + ty - 1) / ty) * nt * B < p.sms;
+  auto pick = [&](auto cb, bool few) {
     constexpr int CB = decltype(cb)::value;
-    if constexpr (sizeof(T) == 4)
-      if (JB > 8) return JB == 12 ? k_idft_mid<T, 12, CB> : k_idft_mid<T, 16, CB>;
-    return JB == 4 ? k_idft_mid<T, 4, CB> : k_idft_mid<T, 8, CB>;
+    if constexpr (sizeof(T) == 4) {
+      if (!few)
+        return wide == 4 ? k_idft_mid<T, 4, CB> : wide == 8 ? k_idft_mid<T, 8, CB>
+             : wide == 12 ? k_idft_mid<T, 12, CB> : k_idft_mid<T, 16, CB>;
+    }
+    return k_idft_mid<T, 4, 1>;
   };
-  // two columns per thread in the z stage, which has N^2 of them per volume; rows of
-  // the y stage are short, one column keeps their CTAs many (11 points: 23 against 33 us)
-  auto midz = pick(std::integral_constant<int, 2>{}), midy = pick(std::integral_constant<int, 1>{});
-  const size_t smem = 2 * cs * (size_t)N * JB;
+  auto midz = pick(std::integral_constant<int, 2>{}, fewz), midy = pick(std::integral_constant<int, 1>{}, fewy);
+  const size_t smz = 2 * cs * (size_t)N * (fewz ? 4 : wide), smy = 2 * cs * (size_t)N * (fewy ? 4 : wide);
   // x stage: Y2[b][tz ty][kx] -> CC[b][tz ty][tx]
   const int rows = nt * nt;
   const size_t smx = cs * (8 * (size_t)N + (size_t)N * nt);
   cudaError_t e;
-  if ((e = allow_smem(midz, smem)) != cudaSuccess || (e = allow_smem(midy, smem)) != cudaSuccess ||
+  if ((e = allow_smem(midz, smz)) != cudaSuccess || (e = allow_smem(midy, smy)) != cudaSuccess ||
       (e = allow_smem(k_idft_x<T>, smx)) != cudaSuccess)
     return e;
-  const int ty = N <= 64 ? 64 : 128;
-  midz<<<dim3((unsigned)((N2 + 255) / 256), 1, B), 128, smem, st>>>(
-      (const C2<T> *)w.Z, (C2<T> *)w.Y1, (const C2<T> *)w.E, N, nt, 1, (int)N2, 2, es);
-  midy<<<dim3((N + ty - 1) / ty, nt, B), ty, smem, st>>>(
-      (const C2<T> *)w.Y1, (C2<T> *)w.Y2, (const C2<T> *)w.E, N, nt, nt, N, 1, es);
+  // FP64: CTAs of two warps, which end more evenly (64 volumes of 24^3, 11 points, z
+  // stage: 139 us with four, 120 with two)
+  const int spz = fewz ? narrow : 1, spy = fewy ? narrow : 1, few_threads = sizeof(T) == 8 ? 64 : 128;
+  const int thz = fewz ? few_threads : 128, colz = fewz ? thz : 256;
+  midz<<<dim3((unsigned)((N2 + colz - 1) / colz * spz), 1, B), thz, smz, st>>>(
+      (const C2<T> *)w.Z, (C2<T> *)w.Y1, (const C2<T> *)w.E, N, nt, 1, (int)N2, 2, es, spz);
+  // (as many threads as columns of a row where the rows make enough CTAs)
+  const int thy = fewy ? few_threads : ty, coly = nt * N;
+  midy<<<dim3((unsigned)((coly + thy - 1) / thy * spy), 1, B), thy, smy, st>>>(
+      (const C2<T> *)w.Y1, (C2<T> *)w.Y2, (const C2<T> *)w.E, N, nt, nt, N, 1, es, spy);
   k_idft_x<T><<<dim3((rows + 7) / 8, B), 256, smx, st>>>(
       (const C2<T> *)w.Y2, (T *)w.CC, (const C2<T> *)w.E, N, nt, rows, T(1.0 / ((double)N2 * N)), es);
   k_cc_argmax<T><<<B, 256, 0, st>>>((const T *)w.CC, nt, org, j0, den, edge, flag_mode, R, t_out,
@@ -789,7 +817,10 @@ cudaError_t launch_shift_search(const Plan &p, const float *f, const float *u, i
   const size_t plane = cs * (2 * (size_t)N * (N | 1) + N);
   if (plane <= 200 * 1024) {
     if ((e = allow_smem(k_fft_plane<T>, plane)) != cudaSuccess) return e;
-    k_fft_plane<T><<<dim3(N, B), 256, plane, st>>>(Z, f, u, fd, tw);
+    // FP64: a thread per radix-4 butterfly at most (64 planes x 16 of 16^2: idle warps'
+    // registers kept other planes off the SM, 49 us with 256 threads, 24 with 64)
+    const int threads = sizeof(T) == 8 ? std::min(256, std::max(64, (N * N / 4 + 31) / 32 * 32)) : 256;
+    k_fft_plane<T><<<dim3(N, B), threads, plane, st>>>(Z, f, u, fd, tw);
   } else {
     // rows, then columns (at least 16, so their rows stay coalesced), about 4096
     // elements per CTA; fewer where they and the twiddles exceed shared memory (FP64
