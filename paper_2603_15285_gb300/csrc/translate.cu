@@ -50,19 +50,57 @@ __device__ __forceinline__ float add_rn(float a, float b) { return __fadd_rn(a, 
 // ---- volume pose ------------------------------------------------------------
 // out_b(x) = vol_b(R_b^T (x - c0) + c0 - s_b), trilinear, zero outside, one
 // thread per output voxel.  R (row-major [B][9]) and s ([B][3]) are nullable
-// (identity, zero).  A CTA takes a brick of 16 x 4 x 4 STEPS voxels, whose rotated
-// corners share cache lines in all directions (a run of 256 along x does not); a
-// thread takes STEPS of them along z, which spreads the block's indices, the pose (its
-// conversion from FP64 runs at that rate) and the rows' products over them.  All index
-// arithmetic is 32-bit: corner indices are clamped next to the box before the
-// conversion (they are outside all the same), the weights keep the unclamped
-// coordinates; one test replaces the eight guards where all corners are inside.  96
-// volumes of 64^3 in FP32: rotated 652 -> 170 us, shifted 266 -> 111 (one voxel per
-// thread 260 and 240; two 208 and 140; four 185 and 122), of which the traffic is 30;
-// then the issue of coordinates and weights.
-constexpr int POSE_X = 16, POSE_Y = 4, POSE_Z = 4;
-template <typename T, int STEPS>
-__global__ void __launch_bounds__(POSE_X * POSE_Y * POSE_Z)
+// (identity, zero).  A thread takes STEPS voxels along z, which spreads the block's
+// indices, the pose (its conversion from FP64 runs at that rate) and the rows' products
+// over them.  All index arithmetic is 32-bit: corner indices are clamped next to the box
+// (they are outside all the same), the weights keep the unclamped coordinates; one test
+// replaces the eight guards where all corners are inside.
+__device__ __forceinline__ int corner_index(float f, int N) {  // -2 .. N + 1 (a NaN gives -2)
+  return (int)fmin(fmax(f, -2.f), (float)(N + 1));
+}
+__device__ __forceinline__ int corner_index(double f, int N) {  // the conversion saturates
+  return min(max(__double2int_rz(f), -2), N + 1);
+}
+template <typename T>
+__device__ __forceinline__ float pose_sample(const float *__restrict__ src, int N, int NN, T px, T py, T pz) {
+  const T fx0 = floor(px), fy0 = floor(py), fz0 = floor(pz);
+  const int i0 = corner_index(fx0, N), j0 = corner_index(fy0, N), k0 = corner_index(fz0, N);
+  const T tx = add_rn(px, -fx0), ty = add_rn(py, -fy0), tz = add_rn(pz, -fz0);
+  float val[8];
+  const unsigned last = N - 1;
+  if ((unsigned)i0 < last && (unsigned)j0 < last && (unsigned)k0 < last) {  // all corners inside
+    const float *p0 = src + (k0 * N + j0) * N + i0, *p1 = p0 + N, *p2 = p0 + NN, *p3 = p1 + NN;
+    val[0] = __ldg(p0); val[1] = __ldg(p0 + 1);
+    val[2] = __ldg(p1); val[3] = __ldg(p1 + 1);
+    val[4] = __ldg(p2); val[5] = __ldg(p2 + 1);
+    val[6] = __ldg(p3); val[7] = __ldg(p3 + 1);
+  } else {
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+      const int ii = i0 + (c & 1), jj = j0 + (c >> 1 & 1), kk = k0 + (c >> 2);
+      val[c] = 0.f;
+      if ((unsigned)ii < (unsigned)N && (unsigned)jj < (unsigned)N && (unsigned)kk < (unsigned)N)
+        val[c] = __ldg(src + (kk * N + jj) * N + ii);
+    }
+  }
+  const T ux = add_rn(T(1), -tx), uy = add_rn(T(1), -ty), uz = add_rn(T(1), -tz);
+  T acc = 0;
+#pragma unroll
+  for (int c = 0; c < 8; ++c) {
+    const T w = mul_rn(mul_rn(c & 1 ? tx : ux, c >> 1 & 1 ? ty : uy), c >> 2 ? tz : uz);
+    acc = add_rn(acc, mul_rn(w, (T)val[c]));
+  }
+  return (float)acc;
+}
+
+// FP32: a CTA takes a brick of 16 x 4 x 4 STEPS voxels, whose rotated corners share
+// cache lines in all directions (a run of 256 along x does not).  96 volumes of 64^3:
+// rotated 652 -> 170 us, shifted 266 -> 111 (one voxel per thread 260 and 240; two 208
+// and 140; four 185 and 122), of which the traffic is 30; then the issue of coordinates
+// and weights.
+constexpr int POSE_X = 16, POSE_Y = 4, POSE_Z = 4, POSE_THREADS = POSE_X * POSE_Y * POSE_Z;
+template <int STEPS>
+__global__ void __launch_bounds__(POSE_THREADS)
 k_pose_volume(int N, int nbx, const float *__restrict__ vol, long vstride,
               const double *__restrict__ R, const double *__restrict__ sh, float *__restrict__ out) {
   const long b = blockIdx.z;
@@ -70,73 +108,89 @@ k_pose_volume(int N, int nbx, const float *__restrict__ vol, long vstride,
   const int i = (blockIdx.x - by * nbx) * POSE_X + threadIdx.x % POSE_X;
   const int j = by * POSE_Y + threadIdx.x / POSE_X % POSE_Y;
   const int kb = blockIdx.y * POSE_Z * STEPS + threadIdx.x / (POSE_X * POSE_Y);
-  __shared__ T r[12];  // R, then s: converted once, conversions from FP64 run at its rate
-  if (threadIdx.x < 9) r[threadIdx.x] = R ? (T)R[9 * b + threadIdx.x] : T(threadIdx.x % 4 == 0);
-  else if (threadIdx.x < 12) r[threadIdx.x] = sh ? (T)sh[3 * b + threadIdx.x - 9] : T(0);
+  __shared__ float r[12];  // R, then s: converted once, conversions from FP64 run at its rate
+  if (threadIdx.x < 9) r[threadIdx.x] = R ? (float)R[9 * b + threadIdx.x] : float(threadIdx.x % 4 == 0);
+  else if (threadIdx.x < 12) r[threadIdx.x] = sh ? (float)sh[3 * b + threadIdx.x - 9] : 0.f;
   __syncthreads();
   if (i >= N || j >= N) return;
   const float *src = vol + b * vstride;
   float *dst = out + b * (long)N * N * N + j * N + i;
-  const T s0 = r[9], s1 = r[10], s2 = r[11];
-  const T c0 = T(0.5) * (T)N;
-  const T x = (T)i - c0, y = (T)j - c0;
+  const float s0 = r[9], s1 = r[10], s2 = r[11];
+  const float c0 = 0.5f * (float)N;
+  const float x = (float)i - c0, y = (float)j - c0;
   // column c of R dotted with (x, y, z), then + c0 - s, left to right
-  const T xy0 = add_rn(mul_rn(r[0], x), mul_rn(r[3], y)), xy1 = add_rn(mul_rn(r[1], x), mul_rn(r[4], y)),
-          xy2 = add_rn(mul_rn(r[2], x), mul_rn(r[5], y));
-  const T r6 = r[6], r7 = r[7], r8 = r[8];
+  const float xy0 = add_rn(mul_rn(r[0], x), mul_rn(r[3], y)), xy1 = add_rn(mul_rn(r[1], x), mul_rn(r[4], y)),
+              xy2 = add_rn(mul_rn(r[2], x), mul_rn(r[5], y));
+  const float r6 = r[6], r7 = r[7], r8 = r[8];
   const int NN = N * N;
 #pragma unroll
   for (int q = 0; q < STEPS; ++q) {
     const int k = kb + q * POSE_Z;
     if (k >= N) break;
-    const T z = (T)k - c0;
-    const T px = add_rn(add_rn(add_rn(xy0, mul_rn(r6, z)), c0), -s0);
-    const T py = add_rn(add_rn(add_rn(xy1, mul_rn(r7, z)), c0), -s1);
-    const T pz = add_rn(add_rn(add_rn(xy2, mul_rn(r8, z)), c0), -s2);
-    const T fx0 = floor(px), fy0 = floor(py), fz0 = floor(pz);
-    // -2 .. N + 1 (a NaN gives -2): past the box on either side with both corners
-    const T lo = T(-2), hi = (T)(N + 1);
-    const int i0 = (int)fmin(fmax(fx0, lo), hi), j0 = (int)fmin(fmax(fy0, lo), hi),
-              k0 = (int)fmin(fmax(fz0, lo), hi);
-    const T tx = add_rn(px, -fx0), ty = add_rn(py, -fy0), tz = add_rn(pz, -fz0);
-    float val[8];
-    const unsigned last = N - 1;
-    if ((unsigned)i0 < last && (unsigned)j0 < last && (unsigned)k0 < last) {  // all corners inside
-      const float *p0 = src + (k0 * N + j0) * N + i0, *p1 = p0 + N, *p2 = p0 + NN, *p3 = p1 + NN;
-      val[0] = __ldg(p0); val[1] = __ldg(p0 + 1);
-      val[2] = __ldg(p1); val[3] = __ldg(p1 + 1);
-      val[4] = __ldg(p2); val[5] = __ldg(p2 + 1);
-      val[6] = __ldg(p3); val[7] = __ldg(p3 + 1);
-    } else {
+    const float z = (float)k - c0;
+    const float px = add_rn(add_rn(add_rn(xy0, mul_rn(r6, z)), c0), -s0);
+    const float py = add_rn(add_rn(add_rn(xy1, mul_rn(r7, z)), c0), -s1);
+    const float pz = add_rn(add_rn(add_rn(xy2, mul_rn(r8, z)), c0), -s2);
+    dst[k * NN] = pose_sample<float>(src, N, NN, px, py, pz);
+  }
+}
+
+// FP64: bound by its pipe, where an operation takes as long for one lane as for 32, so a
+// CTA takes 256 consecutive voxels of a plane, or of the volume where a thread takes
+// one (bricks of 16 leave a quarter of the lanes idle at N = 24), and the clamps work on
+// integers.  64 volumes of 64^3: 2.46 ms before, 2.13 here; of 24^3: 197 us in bricks, 133
+// here.
+template <int STEPS>
+__global__ void __launch_bounds__(POSE_THREADS)
+k_pose_volume64(int N, const float *__restrict__ vol, long vstride, const double *__restrict__ R,
+                const double *__restrict__ sh, float *__restrict__ out) {
+  const long b = blockIdx.z;
+  const int v = blockIdx.x * POSE_THREADS + threadIdx.x, q = v / N, i = v - q * N;
+  const int kb = STEPS == 1 ? q / N : blockIdx.y * STEPS, j = STEPS == 1 ? q - kb * N : q;
+  if (j >= N || kb >= N) return;
+  double r[9], s[3];
 #pragma unroll
-      for (int c = 0; c < 8; ++c) {
-        const int ii = i0 + (c & 1), jj = j0 + (c >> 1 & 1), kk = k0 + (c >> 2);
-        val[c] = 0.f;
-        if ((unsigned)ii < (unsigned)N && (unsigned)jj < (unsigned)N && (unsigned)kk < (unsigned)N)
-          val[c] = __ldg(src + (kk * N + jj) * N + ii);
-      }
-    }
-    const T ux = add_rn(T(1), -tx), uy = add_rn(T(1), -ty), uz = add_rn(T(1), -tz);
-    T acc = 0;
+  for (int c = 0; c < 9; ++c) r[c] = R ? R[9 * b + c] : (c % 4 == 0 ? 1.0 : 0.0);
 #pragma unroll
-    for (int c = 0; c < 8; ++c) {
-      const T w = mul_rn(mul_rn(c & 1 ? tx : ux, c >> 1 & 1 ? ty : uy), c >> 2 ? tz : uz);
-      acc = add_rn(acc, mul_rn(w, (T)val[c]));
-    }
-    dst[k * NN] = (float)acc;
+  for (int c = 0; c < 3; ++c) s[c] = sh ? sh[3 * b + c] : 0.0;
+  const float *src = vol + b * vstride;
+  float *dst = out + b * (long)N * N * N + j * N + i;
+  const double c0 = 0.5 * (double)N, x = (double)i - c0, y = (double)j - c0;
+  // column c of R dotted with (x, y, z), then + c0 - s, left to right
+  const double xy0 = add_rn(mul_rn(r[0], x), mul_rn(r[3], y)), xy1 = add_rn(mul_rn(r[1], x), mul_rn(r[4], y)),
+               xy2 = add_rn(mul_rn(r[2], x), mul_rn(r[5], y));
+  const int NN = N * N;
+#pragma unroll
+  for (int u = 0; u < STEPS; ++u) {
+    const int k = kb + u;
+    if (k >= N) break;
+    const double z = (double)k - c0;
+    const double px = add_rn(add_rn(add_rn(xy0, mul_rn(r[6], z)), c0), -s[0]);
+    const double py = add_rn(add_rn(add_rn(xy1, mul_rn(r[7], z)), c0), -s[1]);
+    const double pz = add_rn(add_rn(add_rn(xy2, mul_rn(r[8], z)), c0), -s[2]);
+    dst[k * NN] = pose_sample<double>(src, N, NN, px, py, pz);
   }
 }
 
 cudaError_t launch_pose_volumes(int N, const float *vol, int B, long vol_stride, const double *R,
                                 const double *shift, bool fp64, float *out, cudaStream_t st) {
   if (B <= 0) return cudaSuccess;
+  if (fp64) {
+    // four voxels per thread where that leaves at most a thirtieth of the lanes idle and
+    // makes six CTAs on each of 152 SMs, whose work then ends evenly; else one
+    const int planes = (N * N + POSE_THREADS - 1) / POSE_THREADS, quads = (N + 3) / 4;
+    if (30L * N * N * N >= 29L * planes * POSE_THREADS * quads * 4 && (long)planes * quads * B >= 912)
+      k_pose_volume64<4><<<dim3(planes, quads, B), POSE_THREADS, 0, st>>>(N, vol, vol_stride, R, shift, out);
+    else
+      k_pose_volume64<1><<<dim3((N * N * N + POSE_THREADS - 1) / POSE_THREADS, 1, B), POSE_THREADS, 0, st>>>(
+          N, vol, vol_stride, R, shift, out);
+    return cudaGetLastError();
+  }
   const int nbx = (N + POSE_X - 1) / POSE_X, nby = (N + POSE_Y - 1) / POSE_Y;
-  constexpr int threads = POSE_X * POSE_Y * POSE_Z;
   auto run = [&](auto steps) {
     constexpr int ST = decltype(steps)::value;
     const dim3 grid((unsigned)(nbx * nby), (unsigned)((N + POSE_Z * ST - 1) / (POSE_Z * ST)), B);
-    if (fp64) k_pose_volume<double, ST><<<grid, threads, 0, st>>>(N, nbx, vol, vol_stride, R, shift, out);
-    else k_pose_volume<float, ST><<<grid, threads, 0, st>>>(N, nbx, vol, vol_stride, R, shift, out);
+    k_pose_volume<ST><<<grid, POSE_THREADS, 0, st>>>(N, nbx, vol, vol_stride, R, shift, out);
   };
   // eight voxels per thread where that still makes four CTAs on each of 152 SMs
   if ((long)nbx * nby * ((N + 31) / 32) * B >= 608) run(std::integral_constant<int, 8>{});

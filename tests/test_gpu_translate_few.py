@@ -1,7 +1,7 @@
-"""GPU tests of the partial inverse transforms where their work is split
-otherwise: few volumes (each group of four grid points on CTAs of its own) and
-FP64 (no padded points, columns packed over the rows), at grids of 1, 4n - 1, 4n
-and 4n + 1 points and boxes that fill no warp."""
+"""GPU tests of the partial inverse transforms and the poses where their work is
+split otherwise: few volumes (each group of four grid points on CTAs of its own)
+and FP64 (no padded points, columns packed over the rows, voxels of a plane in
+runs), at grids of 1, 4n - 1, 4n and 4n + 1 points and boxes that fill no warp."""
 import numpy as np
 import pytest
 import torch
@@ -52,3 +52,23 @@ def test_fp64_values_against_numpy(N, shift, up):
         scale = np.abs(X).sum() / N ** 3
         # FP64: rounding of the transforms and the three sums of N terms
         assert abs(o["cc"][b].item() - cc) <= 1e-13 * scale
+
+
+@pytest.mark.parametrize("prec", [m.FP32, m.FP64])
+@pytest.mark.parametrize("N", [4, 15, 16, 24, 45])
+def test_pose_of_few_and_of_many_volumes(N, prec):
+    """One volume per call (two or one voxels per thread) against many (eight or four)."""
+    B = 2 + 40 * 16 ** 3 * 152 // max(N, 16) ** 3
+    g = torch.Generator(device="cuda").manual_seed(N)
+    v = torch.randn(1, N, N, N, generator=g, device="cuda")
+    R = torch.from_numpy(np.linalg.qr(np.random.default_rng(N).standard_normal((B, 3, 3)))[0]).cuda()
+    s = N * (torch.rand(B, 3, generator=g, device="cuda", dtype=torch.float64) - 0.5)
+    for b, x in enumerate((float("inf"), -float("inf"), float("nan"), 1e300, -1e300, 3e9, -3e9)):
+        s[b, b % 3] = x
+    many = m.matcha_transform_volumes(v, R, s, B=B, precision=prec)
+    for b in (0, 1, 2, 3, 4, 5, 6, 7, 8, B - 1):
+        one = m.matcha_transform_volumes(v, R[b:b + 1].contiguous(), s[b:b + 1].contiguous(), precision=prec)
+        assert torch.equal(one[0].view(torch.int32), many[b].view(torch.int32)), b
+    assert torch.isnan(many[:3]).all()            # positions that are no numbers
+    far = many[3:7] if prec == m.FP64 else many[5:7]  # (1e300 is an infinity in FP32)
+    assert (far == 0).all()
