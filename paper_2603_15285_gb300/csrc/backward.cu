@@ -330,17 +330,20 @@ __device__ __forceinline__ void stage_real(T *dst, const T *src) {
                "l"(src), "n"(sizeof(T)) : "memory");
 }
 
-// A thread's tile of the product is BWD_TS shells x two columns n: per row m (and -m)
-// one 16-byte load of E' and one of each shell's coefficient serve 4 BWD_TS packed
+// A thread's tile of the product is TS shells x two columns n: per row m (and -m)
+// one 16-byte load of E' and one of each shell's coefficient serve 4 TS packed
 // multiply-adds, in the order of m.  The products of a term are fused once and rounded
 // before they are added; which of the two is fused follows the sign of a row's term.
 // Bound by issue (57% of the slots; two barriers per degree): 512 particles of 32
 // shells, L_J = 32, FP32: 468 -> 252 us (4 shells per tile 262, 1 shell slower still).
 // Before, an output's coefficients and E' were read once per product, and the seeds'
 // power loops and a trigonometric function per thread held the block at every degree.
-constexpr int BWD_TS = 2;
+// FP64: one shell, since a tile of few lanes holds a quarter SM as long as a full warp
+// (140 particles of 12 shells, L_J = 16: 54 tiles of two shells on two of the four
+// quarters; with one 196 us, 253 as one output per thread).
+template <typename T> constexpr int BWD_TS = sizeof(T) == 8 ? 1 : 2;
 template <typename T>
-__global__ void __launch_bounds__(BWD_THREADS, sizeof(T) == 4 ? 4 : 2)
+__global__ void __launch_bounds__(BWD_THREADS, sizeof(T) == 4 ? 4 : 3)
     k_bwd_coef(const T *__restrict__ f, int S, int Sc, int L, const double *__restrict__ wrad,
                const T *__restrict__ rcoef, const T *__restrict__ seedK,
                const double *__restrict__ euler, const double *__restrict__ shift,
@@ -445,18 +448,18 @@ __global__ void __launch_bounds__(BWD_THREADS, sizeof(T) == 4 ? 4 : 2)
     //    f_{l,-m} = (-1)^m conj(f_lm) (the sign is in the rows of E')
     const int lm0 = l * (l + 1) / 2, nn = (l + 2) / 2;
     const FastDiv dn(nn);
-    for (int o = threadIdx.x; o < (ns + BWD_TS - 1) / BWD_TS * nn; o += blockDim.x) {
+    for (int o = threadIdx.x; o < (ns + BWD_TS<T> - 1) / BWD_TS<T> * nn; o += blockDim.x) {
       const int st = dn.div(o), n = 2 * (o - st * nn);
-      const T *fq[BWD_TS];
+      const T *fq[BWD_TS<T>];
 #pragma unroll
-      for (int u = 0; u < BWD_TS; ++u) {
-        const int sidx = min(BWD_TS * st + u, ns - 1);
+      for (int u = 0; u < BWD_TS<T>; ++u) {
+        const int sidx = min(BWD_TS<T> * st + u, ns - 1);
         fq[u] = fs + (l & 1) * 2 * Sc * (L + 1) + sidx * 2 * (L + 1);
       }
       const T *ep = Es + 2 * (L * LN + n);
-      P2 xr[BWD_TS], xi[BWD_TS];
+      P2 xr[BWD_TS<T>], xi[BWD_TS<T>];
 #pragma unroll
-      for (int u = 0; u < BWD_TS; ++u) xr[u].x = xr[u].y = xi[u].x = xi[u].y = T(0);
+      for (int u = 0; u < BWD_TS<T>; ++u) xr[u].x = xr[u].y = xi[u].x = xi[u].y = T(0);
       auto rows = [&](int m, auto kind) {  // rows m and -m; kind 0: m = 0, else m's parity
         constexpr int KIND = decltype(kind)::value;
         P2 e0, e1, g0, g1, ne1, ng0;
@@ -467,7 +470,7 @@ __global__ void __launch_bounds__(BWD_THREADS, sizeof(T) == 4 ? 4 : 2)
           ng0.x = -g0.x; ng0.y = -g0.y;
         }
 #pragma unroll
-        for (int u = 0; u < BWD_TS; ++u) {
+        for (int u = 0; u < BWD_TS<T>; ++u) {
           const P2 v = *reinterpret_cast<const P2 *>(fq[u] + 2 * m);
           const T fr = v.x, fi = v.y;
           xr[u] = p_add(xr[u], p_fma(fr, e0, p_mul(fi, ne1)));
@@ -484,8 +487,8 @@ __global__ void __launch_bounds__(BWD_THREADS, sizeof(T) == 4 ? 4 : 2)
         if (m < l) rows(m + 1, std::integral_constant<int, 2>{});
       }
 #pragma unroll
-      for (int u = 0; u < BWD_TS; ++u) {
-        const int sidx = BWD_TS * st + u;
+      for (int u = 0; u < BWD_TS<T>; ++u) {
+        const int sidx = BWD_TS<T> * st + u;
         if (sidx >= ns) break;
         T *xo = Xb + 2L * ((long)sidx * nlm + lm0 + n);
         const T q0 = sc[2 * sidx + (n > 0)], q1 = sc[2 * sidx + 1];
@@ -636,13 +639,22 @@ cudaError_t launch_template_grad(const Plan &p, const T *f, const T *c, int B, i
   const bool vec = (uintptr_t)c % 16 == 0;
   const size_t ps = sizeof(double) * 10 * BWD_THREADS + 2 * sizeof(T) * pw_len(p.LJ);
   auto point = vec ? k_bwd_point<T, true> : k_bwd_point<T, false>;
-  // Shells per CTA: all of them where the batch fills the chip twice over, else split
-  // (each CTA repeats the recurrence); fewer where the coefficients do not fit.
-  int parts = 1;
-  while (2L * parts * BWD_TS <= p.S && (long)B * parts < 2L * p.sms) parts *= 2;
-  int Sc = (p.S + parts - 1) / parts;
-  Sc = (Sc + BWD_TS - 1) / BWD_TS * BWD_TS;
+  // Shells per CTA: each CTA repeats the recurrence, so the shells are split, evenly,
+  // only as far as all CTAs run at once: one on an SM in FP64, whose pipe it fills, two
+  // in FP32 where they fit (twice the CTAs of the chip, whatever the type, cost FP64 130
+  // particles of 24 shells, L_J = 40, 7.51 ms against 2.99 in one part, 76 particles 3.92
+  // against 2.18 in two; FP32 130, L_J = 64, 1.93 against 0.90); more parts where the
+  // coefficients do not fit.
   const size_t most = SMEM_MOST / sizeof(T) - 4;
+  auto shells = [&](long parts) { return (int)(((p.S + parts - 1) / parts + BWD_TS<T> - 1) / BWD_TS<T> * BWD_TS<T>); };
+  auto at_once = [&](long parts) {
+    const size_t bytes = sizeof(T) * (size_t)bwd_coef_reals(p.LJ, shells(parts)) + 2048;
+    return p.sms * (sizeof(T) == 4 && 2 * bytes <= 228 * 1024 ? 2L : 1L);
+  };
+  long parts = 1;
+  while (parts * BWD_TS<T> < p.S && (size_t)bwd_coef_reals(p.LJ, shells(parts)) > most) ++parts;
+  while (2 * parts * BWD_TS<T> <= p.S && 2 * parts * B <= at_once(2 * parts)) parts *= 2;
+  int Sc = shells(parts);
   while (Sc > 1 && (size_t)bwd_coef_reals(p.LJ, Sc) > most) --Sc;
   const size_t smem = sizeof(T) * (size_t)bwd_coef_reals(p.LJ, Sc);
   cudaError_t e = allow_smem(k_bwd_coef<T>, smem, 4 * sizeof(T));
