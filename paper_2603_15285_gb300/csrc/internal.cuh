@@ -40,6 +40,7 @@ struct Plan {
   int tc;        // contraction on the tensor cores: 0 no, 1 TF32, 2 BF16 (FP32 plans)
   int *dev_err;  // device word: bit 0 = a tensor-core wait reached its limit
   int sms = 1;                     // SMs of that device
+  int clusters[4][10] = {};        // [r - 1][q]: clusters_at_once
   int device = -1;                 // the CUDA device current at plan creation
   void *noalloc_grid = nullptr;    // device address of the allocation-free search's array
   // tile choices set by matcha_plan_autotune (0 = the built-in rule); none of
@@ -101,6 +102,13 @@ struct Plan {
 };
 void destroy_texsets(Plan &p);
 
+// Clusters of q <= 9 CTAs that run at once where r CTAs fit an SM.  A cluster stays
+// within one group of SMs, and the groups' sizes do not divide evenly: of 152 SMs with
+// one CTA each, 46 clusters of three run at once, not 50, 36 of four, 15 of eight.
+inline long clusters_at_once(const Plan &p, int r, int q) {
+  return r <= 4 ? p.clusters[r - 1][q] : (long)p.clusters[3][q] * r / 4;
+}
+
 inline size_t align_up(size_t x, size_t a = 256) { return (x + a - 1) / a * a; }
 
 // Opts a kernel in to a launch with `bytes` of dynamic shared memory; `fixed` is the
@@ -151,13 +159,16 @@ inline long pair_entries_host(int L) {  // sum_{m<=L} (2m+1)(L-m+1)
 
 // Table builders (plan_tables.cu).
 cudaError_t build_tables(Plan &p, cudaStream_t st);
+void count_clusters(Plan &p);  // p.clusters
 // The ball-harmonic radial table on the host (ball.cu): W[l][k][s] =
 // w_s N_lk j_l(lambda_lk r_s / R) for k < |K_l| (zero-padded to Kmax), the
 // counts |K_l|; returns Kmax = |K_0|.
 int ball_tables(int L, int S, double R, double Lam, const double *r, const double *w,
                 std::vector<double> &W, std::vector<int> &counts);
 
-// Kernel launchers; each returns cudaGetLastError() after its launches.
+// Kernel launchers; each returns cudaGetLastError() after its launches.  batch: the
+// particles of a call whose parts run on several streams at once (0: B), which decides
+// whether a launch may spread over idle SMs.
 template <typename T>
 cudaError_t launch_analyze(const Plan &p, const float *vols, int B, T *coef, cudaStream_t st,
                            const float *vols2 = nullptr, int B2 = 0, T *coef2 = nullptr);
@@ -166,10 +177,10 @@ cudaError_t launch_correlate(const Plan &p, const T *f, const T *h, int B, int h
                              cudaStream_t st);
 template <typename T>
 cudaError_t launch_soft(const Plan &p, const T *c, int B, const int *P_per, T *grid, int *idx,
-                        double *euler, double *score, int *n_cand, cudaStream_t st);
+                        double *euler, double *score, int *n_cand, cudaStream_t st, int batch = 0);
 template <typename T>
 cudaError_t launch_newton(const Plan &p, const T *c, int B, const int *n_cand, double *euler,
-                          double *score, int *cflags, long long *work, cudaStream_t st);
+                          double *score, int *cflags, long long *work, cudaStream_t st, int batch = 0);
 template <typename T>
 cudaError_t launch_newton_queue(const Plan &p, const T *c, int B, const int *n_cand, double *euler,
                                 double *score, int *cflags, long long *work, int *order,
@@ -190,7 +201,7 @@ size_t newton_smem(const Plan &p);                // of one CTA per particle
 bool newton_rescaled(const Plan &p);              // the rescaled 32-bit recurrence runs
 int newton_schedule(const Plan &p, std::vector<int4> &out);  // returns the rounds
 template <typename T>  // false: not launched, one CTA per particle is as fast
-bool launch_newton_spread(const Plan &p, const T *c, int B, const int *n_cand, double *euler,
+bool launch_newton_spread(const Plan &p, const T *c, int B, int batch, const int *n_cand, double *euler,
                           double *score, int *cflags, long long *work, cudaStream_t st, cudaError_t *e);
 template <typename T>
 bool launch_objective_spread(const Plan &p, const T *c, int B, int L, int Q, const double *pts,

@@ -203,6 +203,7 @@ matcha_status matcha_plan_create(const matcha_plan_desc *d, matcha_plan *out) {
   if (e != cudaSuccess) { delete p; return fail_cuda(e, "cudaGetDevice"); }
   cudaDeviceGetAttribute(&p->sms, cudaDevAttrMultiProcessorCount, p->device);
   if (p->sms <= 0) p->sms = 1;
+  count_clusters(*p);
   e = cudaMalloc(&p->base, sz);
   if (e != cudaSuccess) { delete p; return fail_cuda(e, "cudaMalloc(plan tables)"); }
   char *b = (char *)p->base;
@@ -455,11 +456,11 @@ matcha_status matcha_final_select(matcha_plan plan, int B, const int *P_per, con
 
 // Steps a1..a7 for the particle range covered by `w` (workspace arrays already
 // offset to the range's first particle); the templates' coefficients are
-// analysed here unless `h_ready`.
+// analysed here unless `h_ready`.  batch: particles of all ranges in flight.
 static matcha_status align_range(matcha_plan plan, const float *particles, const float *templates,
                                  int B, int tstride, bool h_ready, const int *P_per, double *euler,
                                  double *R, double *score, int *best_p, int *flags,
-                                 const AlignWs &w, void *stream) {
+                                 const AlignWs &w, int batch, void *stream) {
   Plan *p = P_(plan);
   const int Bt = tstride ? B : 1;
   matcha_status s;
@@ -484,9 +485,9 @@ static matcha_status align_range(matcha_plan plan, const float *particles, const
     cudaStream_t st = (cudaStream_t)stream;
     cudaError_t e = p->fp64 ? launch_soft<double>(*p, (const double *)w.c, B, P_per,
                                                   (double *)w.grid, w.cidx, w.ceuler, w.cscore,
-                                                  w.ncand, st)
+                                                  w.ncand, st, batch)
                             : launch_soft<float>(*p, (const float *)w.c, B, P_per, (float *)w.grid,
-                                                 w.cidx, w.ceuler, w.cscore, w.ncand, st);
+                                                 w.cidx, w.ceuler, w.cscore, w.ncand, st, batch);
     if (e != cudaSuccess) return fail_cuda(e, "soft_search");
   }
   {
@@ -500,9 +501,12 @@ static matcha_status align_range(matcha_plan plan, const float *particles, const
                                                            w.ceuler, w.cscore, w.cflags, nullptr,
                                                            w.order, w.ticket, st);
       if (e != cudaSuccess) return fail_cuda(e, "newton_march");
-    } else if ((s = matcha_newton_march(plan, w.c, B, w.ncand, w.ceuler, w.cscore, w.cflags,
-                                        nullptr, stream))) {
-      return s;
+    } else {
+      cudaError_t e = p->fp64 ? launch_newton<double>(*p, (const double *)w.c, B, w.ncand, w.ceuler, w.cscore,
+                                                      w.cflags, nullptr, st, batch)
+                              : launch_newton<float>(*p, (const float *)w.c, B, w.ncand, w.ceuler, w.cscore,
+                                                     w.cflags, nullptr, st, batch);
+      if (e != cudaSuccess) return fail_cuda(e, "newton_march");
     }
   }
   Range r("a7 final selection");
@@ -547,7 +551,7 @@ matcha_status matcha_align(matcha_plan plan, const float *particles, const float
   // (large L0: its grid and scan kernels gain nothing from the split)
   if (B < 256 || !soft_grid_optional(*p))
     return align_range(plan, particles, templates, B, tstride, false, P_per, euler, R, score,
-                       best_p, flags, w, stream);
+                       best_p, flags, w, B, stream);
   // Parts of at least 128 particles on up to NSPLIT streams (the caller's and
   // ones the plan owns), joined back into the caller's stream: each part's
   // kernels fill the others' wave tails.  Every particle's arithmetic is the
@@ -586,7 +590,7 @@ matcha_status matcha_align(matcha_plan plan, const float *particles, const float
     const AlignWs wk = ws_at(*p, w, b0, tstride);
     s = align_range(plan, particles + vox * b0, tstride ? templates + vox * b0 : templates,
                     b1 - b0, tstride, h_ready, P_per ? P_per + b0 : nullptr, euler + 3 * b0,
-                    R + 9 * b0, score + b0, best_p + b0, flags + b0, wk, sk);
+                    R + 9 * b0, score + b0, best_p + b0, flags + b0, wk, B, sk);
     if (k) {
       cudaError_t e = cudaEventRecord(p->ev_join[k - 1], sk);
       if (e != cudaSuccess) {

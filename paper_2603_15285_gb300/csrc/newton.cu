@@ -833,10 +833,10 @@ bool newton_fits(const Plan &p) { return newton_slots(p) > 0; }
 
 template <typename T>
 cudaError_t launch_newton(const Plan &p, const T *c, int B, const int *n_cand, double *euler,
-                          double *score, int *cflags, long long *work, cudaStream_t st) {
+                          double *score, int *cflags, long long *work, cudaStream_t st, int batch) {
   if (B == 0) return cudaSuccess;
   cudaError_t e;
-  if (launch_newton_spread<T>(p, c, B, n_cand, euler, score, cflags, work, st, &e)) return e;
+  if (launch_newton_spread<T>(p, c, B, std::max(B, batch), n_cand, euler, score, cflags, work, st, &e)) return e;
   NewtonArgs A;
   A.LJ = p.LJ; A.nlev = p.nlev; A.M = p.M; A.P = p.P;
   A.cpw = newton_cpw(p.P);
@@ -933,9 +933,9 @@ template cudaError_t launch_objective<double>(const Plan &, const double *, int,
                                               const double *, double *, cudaStream_t);
 
 template cudaError_t launch_newton<float>(const Plan &, const float *, int, const int *, double *,
-                                          double *, int *, long long *, cudaStream_t);
+                                          double *, int *, long long *, cudaStream_t, int);
 template cudaError_t launch_newton<double>(const Plan &, const double *, int, const int *, double *,
-                                           double *, int *, long long *, cudaStream_t);
+                                           double *, int *, long long *, cudaStream_t, int);
 
 // Eight lanes per particle: the candidates' scores and flags are read together and
 // three lanes take one angle's sincos each.  (A thread per particle: 10.5 us for one

@@ -810,11 +810,16 @@ size_t spread_smem(const Plan &p, size_t tsize, SpreadArgs &A) {
 //
 // 32-bit plans: several workers per chain group, worth it only while SMs are
 // idle.  In units of one CTA per particle alone on its SM, W workers take
-// t(W) = a + (1 - a) / W, where a, the share of the tables and the step rule,
-// falls with the entries per sub-slot (480 / (480 + entries): 8 particles to
-// L = 32: 478 us, W = 4 341, W = 8 289; 36 to L = 100: 6.26 ms, 1.80, 1.21); more
-// than one such CTA per SM costs a quarter more.  One CTA per particle takes 1 per
-// wave of one CTA per SM and 1.5 with two (96 and 304 particles: 500, 760 us).
+// a + f (1 - a) / W, where a, the share of the tables and the step rule, falls
+// with the entries per sub-slot (560 / (700 + entries)) and f is 1.3 with eight
+// warps on an SM, 1.6 with sixteen (eight particles of 16 candidates: to L = 16 141 us,
+// W = 4 119, W = 8 114; L = 32 242, 153, 138; L = 64 822, 332, 245; L = 100 8.73 ms,
+// 2.50, 1.58).  One CTA per particle takes 1 per wave of one CTA per SM and 1.5
+// with two (96 and 304 particles: 500, 760 us).
+//
+// A wave holds as many clusters as run at once (clusters_at_once), not its share of the
+// SMs: 76 particles to L = 48 in clusters of four, two waves of SMs but three of
+// clusters, took 653 us against 448 as single CTAs.
 bool spread_shape(const Plan &p, size_t tsize, int B, SpreadArgs &out, size_t *smem) {
   SpreadArgs A = {};
   A.LJ = p.LJ; A.nlev = p.nlev; A.M = p.M; A.P = p.P;
@@ -829,7 +834,7 @@ bool spread_shape(const Plan &p, size_t tsize, int B, SpreadArgs &out, size_t *s
   A.pairs = p.P <= 16;
   const bool fp64 = tsize == 8;
   const long sm_bytes = 228 * 1024, most = 227 * 1024, reg_warps = fp64 ? 8 : 16, sms = p.sms;
-  const double entries = (double)p.nc / 2 / A.nslots, a = 480 / (480 + entries);
+  const double entries = (double)p.nc / 2 / A.nslots, a = 560 / (700 + entries);
   const long one = std::max(1L, std::min<long>(sm_bytes / (long)(newton_smem(p) + 1024), reg_warps / 8));
   double best = fp64 ? 1e30 : 0.95 * (B <= sms ? 1 : ((B + one * sms - 1) / (one * sms)) * (one > 1 ? 1.5 : 1));
   bool found = false;
@@ -847,10 +852,10 @@ bool spread_shape(const Plan &p, size_t tsize, int B, SpreadArgs &out, size_t *s
       }
       if ((long)bytes > most) continue;
       const long resident = std::max(1L, std::min<long>(sm_bytes / (long)(bytes + 1024), reg_warps / (cpc * W)));
-      const long n = (long)B * A.ctas, waves = (n + resident * sms - 1) / (resident * sms);
-      const long per_sm = std::min(resident, (n + sms - 1) / sms);
+      const long n = (long)B * A.ctas, held = clusters_at_once(p, (int)resident, A.ctas), waves = (B + held - 1) / held;
+      const long per_sm = std::min(resident, (n + sms - 1) / sms), warps = per_sm * cpc * W;
       const double t = fp64 ? waves * std::max(4.0, (double)per_sm * cpc)
-                            : waves * (a + (1 - a) / W) * (per_sm > 1 ? 1.25 : 1);
+                            : waves * (a + (1 - a) / W * (warps > 8 ? 1.6 : warps > 4 ? 1.3 : 1));
       if (t < best) {
         best = t;
         out = A;
@@ -908,11 +913,11 @@ int newton_schedule(const Plan &p, std::vector<int4> &out) {
 
 // False when one CTA per particle is expected to be as fast.
 template <typename T>
-bool launch_newton_spread(const Plan &p, const T *c, int B, const int *n_cand, double *euler,
+bool launch_newton_spread(const Plan &p, const T *c, int B, int batch, const int *n_cand, double *euler,
                           double *score, int *cflags, long long *work, cudaStream_t st, cudaError_t *e) {
   SpreadArgs A;
   size_t smem;
-  if (!spread_shape(p, sizeof(T), B, A, &smem)) return false;
+  if (!spread_shape(p, sizeof(T), batch, A, &smem)) return false;
   auto kern = A.W > 1 ? k_newton_spread<T, false, true> : k_newton_spread<T, false, false>;
   if constexpr (sizeof(T) == 4)
     if (newton_rescaled(p)) kern = A.W > 1 ? k_newton_spread<T, true, true> : k_newton_spread<T, true, false>;
@@ -920,9 +925,9 @@ bool launch_newton_spread(const Plan &p, const T *c, int B, const int *n_cand, d
                        score, cflags, work);
   return true;
 }
-template bool launch_newton_spread<float>(const Plan &, const float *, int, const int *, double *,
+template bool launch_newton_spread<float>(const Plan &, const float *, int, int, const int *, double *,
                                           double *, int *, long long *, cudaStream_t, cudaError_t *);
-template bool launch_newton_spread<double>(const Plan &, const double *, int, const int *, double *,
+template bool launch_newton_spread<double>(const Plan &, const double *, int, int, const int *, double *,
                                            double *, int *, long long *, cudaStream_t, cudaError_t *);
 
 template <typename T>

@@ -13,6 +13,9 @@
 //   e  = (l+1) Q_l / (l Q_{l+1}),  Q_j = sqrt((j^2 - m^2)(j^2 - n^2)),
 // seeded at l = m >= |n| by d^m_{mn} = sqrt(C(2m, m+n)) cos(b/2)^{m+n} (-sin(b/2))^{m-n}.
 #include <math.h>
+#include <algorithm>
+#include <array>
+#include <map>
 #include "internal.cuh"
 
 namespace matcha {
@@ -253,6 +256,43 @@ __global__ void k_transpose(int ns, long n, const T *in, T *out) {
   const long t = blockIdx.x * (long)blockDim.x + threadIdx.x;
   if (t >= n * ns) return;
   out[t] = in[(t % ns) * n + t / ns];
+}
+
+__global__ void k_cluster_probe() {}
+
+// As the driver counts them for a kernel that only shared memory limits; a property of
+// the device, so asked once per device.
+void count_clusters(Plan &p) {
+  static std::mutex mu;
+  static std::map<int, std::array<int, 40>> known;
+  std::lock_guard<std::mutex> lock(mu);
+  auto at = known.find(p.device);
+  if (at == known.end()) {
+    std::array<int, 40> n{};
+    bool asked = allow_smem(k_cluster_probe, SMEM_MOST) == cudaSuccess &&
+                 cudaFuncSetAttribute(k_cluster_probe, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
+    for (int r = 1; r <= 4; ++r)
+      for (int q = 1; q < 10; ++q) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(q);
+        cfg.blockDim = dim3(32);
+        cfg.dynamicSmemBytes = 228 * 1024 / r - 1024;
+        cudaLaunchAttribute a;
+        a.id = cudaLaunchAttributeClusterDimension;
+        a.val.clusterDim.x = q;
+        a.val.clusterDim.y = a.val.clusterDim.z = 1;
+        cfg.attrs = &a;
+        cfg.numAttrs = 1;
+        int v = 0;
+        if (!asked || cudaOccupancyMaxActiveClusters(&v, k_cluster_probe, &cfg) != cudaSuccess || v < 1)
+          v = std::max(1, r * p.sms / (q + 1));  // not told: fewer than an even share
+        n[10 * (r - 1) + q] = q == 1 ? r * p.sms : v;
+      }
+    cudaGetLastError();
+    at = known.emplace(p.device, n).first;
+  }
+  for (int r = 0; r < 4; ++r)
+    for (int q = 1; q < 10; ++q) p.clusters[r][q] = at->second[10 * r + q];
 }
 
 cudaError_t build_tables(Plan &p, cudaStream_t st) {

@@ -1256,8 +1256,9 @@ static cudaError_t launch_clusters(K kern, int B, int CL, int threads, size_t sm
 
 template <typename T>
 cudaError_t launch_soft(const Plan &p, const T *c, int B, const int *P_per, T *grid, int *idx,
-                        double *euler, double *score, int *n_cand, cudaStream_t st) {
+                        double *euler, double *score, int *n_cand, cudaStream_t st, int batch) {
   if (B == 0) return cudaSuccess;
+  batch = std::max(B, batch);
   // the warp-per-slice kernel only when chosen (autotuner or matcha_plan_set_tiles):
   // measured slower than the chunked kernel at L0 = 8, K = 2 (0.43 against 0.16 ms
   // for 256 particles)
@@ -1272,9 +1273,11 @@ cudaError_t launch_soft(const Plan &p, const T *c, int B, const int *P_per, T *g
   }
   // the register-tiled kernel unless another was chosen (bit-identical to the chunked one)
   if (sizeof(T) == 4 && (p.tune_soft == 0 || p.tune_soft == 3) && soft_tile_ok(p)) {
-    // a particle over nine CTAs (a pass each) while each has an SM (1 particle: 82 us on
-    // one CTA, 24), over three while two share one (96 particles: 93 us, 62)
-    const int CL = 9L * B <= p.sms ? SOFT_SPLIT_MOST : 3L * B <= 2L * p.sms ? 3 : 1;
+    // a particle over nine CTAs (a pass each) while all run with an SM each (1 particle:
+    // 82 us on one CTA, 24), over three while two share one (96 particles: 93 us, 62)
+    const int CL = batch <= clusters_at_once(p, 1, SOFT_SPLIT_MOST) ? SOFT_SPLIT_MOST
+                 : batch <= clusters_at_once(p, 2, 3)               ? 3
+                                                                    : 1;
     const size_t smem = soft_tile_smem(p, CL > 1);
     auto kern = CL == 9 ? k_soft_split<TILE_KB, 8, 36, SOFT_SPLIT_MOST>
               : CL == 3 ? k_soft_split<TILE_KB, 8, 36, 3> : k_soft_tile<TILE_KB, 8, 36>;
@@ -1290,17 +1293,20 @@ cudaError_t launch_soft(const Plan &p, const T *c, int B, const int *P_per, T *g
       auto kern = k_soft_chunk<T, SOFT_KB>;
       const cudaError_t e = allow_smem(kern, smem);
       if (e != cudaSuccess) return e;
-      // CTAs per particle: passes of the longest one (and the short one ahead) times the
-      // waves; two CTAs on an SM take a third longer.  40 particles in FP64, 36 points
-      // per angle: 829 us on one CTA each, 337 on three.
+      // CTAs per particle: the passes of one and its setup (one or two passes' time) times the waves of clusters that run at once; two CTAs on an SM take a
+      // quarter longer.  40 particles in FP64, 36 points per angle: 829 us on one CTA
+      // each, 337 on three; 100 particles: 823 on one, 978 on three (46 clusters of three
+      // at once, so three waves).  FP32, 42 points: 16 particles 124 us on one, 46 on
+      // six; 50 particles 128, 81 on two (117 on three); 100 particles 131 (169 on three).
       const int passes = (p.ns + SOFT_KB - 1) / SOFT_KB, one = sizeof(T) == 8 || 2 * (smem + 1024) > 228 * 1024 ? 1 : 2;
+      const double setup = sizeof(T) == 8 ? 1.2 : 1.6;
       int CL = 1;
       double best = 1e30;
       for (int q = 1; q <= std::min(8, passes); ++q) {
         if (q > 1 && (passes + q - 1) / q * (q - 1) >= passes) continue;  // a CTA without slices
-        const long n = (long)B * q, waves = (n + one * p.sms - 1) / (one * p.sms);
-        const double t = waves * ((passes + q - 1) / q + (q > 1 ? 0.6 : 0.0)) * (n > p.sms && one > 1 ? 1.33 : 1.0);
-        if (t < 0.95 * best) { best = t; CL = q; }
+        const long held = clusters_at_once(p, one, q), waves = (batch + held - 1) / held;
+        const double t = waves * ((passes + q - 1) / q + setup) * ((long)batch * q > p.sms && one > 1 ? 1.25 : 1.0);
+        if (t < 0.97 * best) { best = t; CL = q; }
       }
       return launch_clusters(kern, B, CL, CHUNK_THREADS, smem, st, c, p.nc, p.L0, p.ns, p.pair_base,
                              (const T *)p.soft_d, p.pair_off0, p.nc0, (const T *)p.soft_tw, p.P, P_per, grid,
@@ -1321,8 +1327,8 @@ cudaError_t launch_soft(const Plan &p, const T *c, int B, const int *P_per, T *g
 }
 
 template cudaError_t launch_soft<float>(const Plan &, const float *, int, const int *, float *, int *,
-                                        double *, double *, int *, cudaStream_t);
+                                        double *, double *, int *, cudaStream_t, int);
 template cudaError_t launch_soft<double>(const Plan &, const double *, int, const int *, double *,
-                                         int *, double *, double *, int *, cudaStream_t);
+                                         int *, double *, double *, int *, cudaStream_t, int);
 
 }  // namespace matcha
