@@ -169,11 +169,17 @@ __host__ __device__ __forceinline__ long slab_reals(int L0, int ns, int KS, int 
 // pairs and whose rows and columns are two quads half the padded range apart,
 // so that the lanes of a 16-byte shared load read consecutive quads.  As many
 // slices share a CTA as give its 256 threads one tile each.
+// FP64 is bound by its pipe, an operation holding a quarter SM as long for one lane as
+// for 32, so stage 2 items are one pair of rows x one gamma there, enough for all warps
+// (four rows x four gammas at 52 points: 52 items on two of the four quarters), and two
+// CTAs share an SM, one's arithmetic over the other's barriers.  140 particles at 52
+// points: 5.35 ms -> 3.02 (4.46 streamed on one CTA per particle).
 template <typename T>
-__global__ void __launch_bounds__(256, sizeof(T) == 8 ? 1 : 2)
+__global__ void __launch_bounds__(256, 2)
 k_soft_slab(int L0, int ns, int KS, int IC, const T *__restrict__ tw, T *__restrict__ grid, int vec) {
   typedef typename Pair<T>::type P2;
   constexpr int TI = Tile<T>::I, TJ = Tile<T>::J, QI = TI / 4, QJ = TJ / 4;
+  constexpr int SV = sizeof(T) == 8 ? 1 : 2, SU = sizeof(T) == 8 ? 1 : 4;  // stage 2 item: row pairs, gammas
   const long b = blockIdx.y;
   const int k0 = blockIdx.x * KS, nk = min(KS, ns - k0);
   const int W = 2 * L0 + 1, M1 = L0 + 1, MP = slab_pairs(L0), NJ = round_up(ns, TJ);
@@ -251,38 +257,38 @@ k_soft_slab(int L0, int ns, int KS, int IC, const T *__restrict__ tw, T *__restr
   }
   __syncthreads();
   {
-    const int jt = NJ / 4, mt = MP / 2;
+    const int jt = NJ / SU, mt = ((M1 + 1) / 2 + SV - 1) / SV;
     const FastDiv djt(jt), dmt(mt);
     for (int t = tid; t < nk * mt * jt; t += NT) {
       const int km = djt.div(t), jq = t - km * jt, kk = dmt.div(km), mq = km - kk * mt;
-      int tt[4], js[4];
+      int tt[SU], js[SU];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
+      for (int u = 0; u < SU; ++u) {
         const int j = jq + u * jt;
         js[u] = j < ns ? j : 0;  // columns of the padding are computed as column 0, never stored
         const int lj = L0 * js[u], r = lj - dns.div(lj) * ns;
         tt[u] = r ? ns - r : 0;  // (-L0 j) mod ns
       }
-      P2 re[2][4], im[2][4];
+      P2 re[SV][SU], im[SV][SU];
 #pragma unroll
-      for (int v = 0; v < 2; ++v)
+      for (int v = 0; v < SV; ++v)
 #pragma unroll
-        for (int u = 0; u < 4; ++u) re[v][u] = im[v][u] = pdup(T(0));
-      const T *row = Sp + ((long)kk * W * MP + 2 * mq) * 4;
+        for (int u = 0; u < SU; ++u) re[v][u] = im[v][u] = pdup(T(0));
+      const T *row = Sp + ((long)kk * W * MP + SV * mq) * 4;
       for (int n = 0; n < W; ++n, row += 4 * MP) {
-        P2 sr[2], si[2];
+        P2 sr[SV], si[SV];
 #pragma unroll
-        for (int v = 0; v < 2; ++v) {
+        for (int v = 0; v < SV; ++v) {
           const Quad<T> s = *reinterpret_cast<const Quad<T> *>(row + 4 * v);
           sr[v] = pset(s.v[0], s.v[1]);
           si[v] = pset(s.v[2], s.v[3]);
         }
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
+        for (int u = 0; u < SU; ++u) {
           const P2 e = *reinterpret_cast<const P2 *>(tws + 2 * tt[u]);
           const P2 cr = pdup(e.x), ci = pdup(e.y), ni = pdup(-e.y);
 #pragma unroll
-          for (int v = 0; v < 2; ++v) {
+          for (int v = 0; v < SV; ++v) {
             re[v][u] = padd(re[v][u], pfma(sr[v], cr, pmul(si[v], ni)));
             im[v][u] = padd(im[v][u], pfma(sr[v], ci, pmul(si[v], cr)));
           }
@@ -291,14 +297,14 @@ k_soft_slab(int L0, int ns, int KS, int IC, const T *__restrict__ tw, T *__restr
         }
       }
 #pragma unroll
-      for (int v = 0; v < 2; ++v)
+      for (int v = 0; v < SV; ++v)
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-          const int m = 4 * mq + 2 * v + h;
+          const int m = 2 * (SV * mq + v) + h;
           if (m >= M1) continue;
           T *o = G + ((long)kk * M1 + m) * 2 * NJ + jq;
 #pragma unroll
-          for (int u = 0; u < 4; ++u) {
+          for (int u = 0; u < SU; ++u) {
             o[u * jt] = h ? re[v][u].y : re[v][u].x;
             o[NJ + u * jt] = h ? im[v][u].y : im[v][u].x;
           }
