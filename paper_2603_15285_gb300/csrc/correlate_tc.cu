@@ -706,21 +706,27 @@ cudaError_t launch_correlate_tc(const Plan &p, const float *f, const float *h, i
   const int bf16 = p.tc == 2;
   const TcGeom g = tc_geom(p.S, p.LJ, bf16 ? 2 : 4);
   if (!correlate_tc_fits(p.S, p.LJ, bf16 ? 2 : 4) || p.S > 128) return cudaErrorInvalidConfiguration;
-  static int nsm = 0;
-  if (!nsm) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    if (nsm <= 0) nsm = 1;
-  }
+  const int nsm = p.sms;
   const int PM = hstride ? 0 : tc_shared_stack(g, p.S, p.LJ);
-  if (PM) {
-    // particles per block: B's staging is shared by more of them (8: 387 us, 16: 351 us at
-    // the size above; at most 16: the blocks in flight then write about 64 MB, so that the
-    // degrees of an output line meet in L2) while there are four units per SM
-    int PB = PM;
-    while (PB < 16 && (long)((B + 2 * PB - 1) / (2 * PB)) * (p.LJ / 2 + 1) >= 4L * nsm) PB *= 2;
-    const long units = (long)((B + PB - 1) / PB) * (p.LJ / 2 + 1);
+  // Particles per block: their passes share one staging of B, worth about 2.5 particles,
+  // but the blocks have to fill the SMs (at most 16: those in flight then write about 64
+  // MB, so that the degrees of an output line meet in L2).  An item of k_correlate_tc, two
+  // on an SM, takes about as long as 4.2 particles of a pass.  768 particles, 32 shells,
+  // L_J = 48, TF32: 387 us with 8, 351 with 16; 17 and 64 particles, 24 shells, L_J = 33:
+  // 14 and 31 us with k_correlate_tc, 20 and 34 in blocks of two, 17 and 23 in blocks of
+  // four and eight.
+  const int pairs = p.LJ / 2 + 1;
+  const long items = (long)B * pairs;
+  int PB = 0;
+  double best = 1e30;
+  for (int q = PM; q && q <= 16; q *= 2) {
+    const long units = (long)((B + q - 1) / q) * pairs;
+    const double t = (units + nsm - 1) / nsm * (2.5 + q);
+    if (t < best) { best = t; PB = q; }
+  }
+  const bool shared = PB && items > 2L * nsm && best <= 4.2 * ((items + 2L * nsm - 1) / (2L * nsm));
+  if (shared) {
+    const long units = (long)((B + PB - 1) / PB) * pairs;
     const int smem1 = (int)tc_shared(g, p.LJ, PM).smem;
     const long limit = p.wait_limit >= 0 ? p.wait_limit : TC_WAIT_LIMIT;
     auto kern = bf16 ? k_correlate_tc_shared<1> : k_correlate_tc_shared<0>;
@@ -730,7 +736,6 @@ cudaError_t launch_correlate_tc(const Plan &p, const float *f, const float *h, i
                                                                       PB, PM, p.dev_err, limit);
     return cudaGetLastError();
   }
-  const long items = (long)B * (p.LJ / 2 + 1);
   const long per_sm = p.tune_tc_ctas == 1 ? 1 : 2;
   const int grid = (int)(items < per_sm * nsm ? items : per_sm * nsm);
   const size_t smem = (size_t)tc_smem(g);
