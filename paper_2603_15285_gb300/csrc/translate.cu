@@ -585,14 +585,15 @@ template <> struct CPair<float> { typedef float2 type; typedef float4 quad; };
 template <> struct CPair<double> { typedef double2 type; typedef Double4 quad; };
 
 // out[b][a][j][c] = sum_k in[b][a][k][c] E[b][axis][k][j]: the partial inverse
-// DFT along a middle (y) or outer (z) axis.  A thread takes CB of the A C columns (a, c)
-// of a particle, JB grid points j at a time in registers against the factors in shared
-// memory (one 16-byte broadcast per CB products of three packed operations); four rows
-// k of its columns are in flight while the four before are multiplied.  SP CTAs share a
-// tile of columns, each with every SP-th group of JB points.  es: elements between the
-// particles' factors (0: shared).
+// DFT along a middle (y) or outer (z) axis.  A thread takes CB columns c, JB grid
+// points j at a time in registers against the factors in shared memory (one 16-byte
+// broadcast per CB products of three packed operations); four rows k of its columns
+// are in flight while the four before are multiplied.  PACK: one of the A C columns (a,
+// c), and SP CTAs share a tile of them, each with every SP-th group of JB points (else
+// the rows a are CTAs' and SP is 1).  es: elements between the particles' factors (0:
+// shared).
 //
-// FP32, SP = 1: 96 volumes of 64^3, 11 and 29 grid points: the z stage 139 and 171 us
+// FP32, many volumes: 96 volumes of 64^3, 11 and 29 grid points: the z stage 139 and 171 us
 // -> 76 and 97 (one column per thread 97 and 117; two without the loads ahead 128 and
 // 143), then bound by its FMAs (floor 33) and, past 16 points, by reading the volume
 // again.  One volume, 41 points: 41 and 40 us in the z and y stages on 16 and 41 CTAs;
@@ -602,7 +603,7 @@ template <> struct CPair<double> { typedef double2 type; typedef Double4 quad; }
 // are packed into warps; one column, four points and a CTA per group of points spread the
 // work evenly.  64 volumes of 64^3, 41 points: 7.5 and 4.8 ms (eight padded points, two
 // columns in the z stage: 9.0 and 5.8); one volume: 165 and 112 us (1,304 and 633).
-template <typename T, int JB, int CB>
+template <typename T, int JB, int CB, bool PACK>
 __global__ void __launch_bounds__(128)
 k_idft_mid(const C2<T> *__restrict__ in, C2<T> *__restrict__ out, const C2<T> *__restrict__ E,
            int N, int nt, int A, int C, int axis, long es, int SP) {
@@ -611,19 +612,19 @@ k_idft_mid(const C2<T> *__restrict__ in, C2<T> *__restrict__ out, const C2<T> *_
   extern __shared__ __align__(16) unsigned char smem_raw[];
   Q *Es = reinterpret_cast<Q *>(smem_raw);  // [N][JB]
   const long b = blockIdx.z;
-  const int tile = blockIdx.x / SP, tid = threadIdx.x, cols = A * C;
-  const P2 *src[CB];
-  P2 *dst[CB];
+  static_assert(!PACK || CB == 1, "packed columns are single");
+  const int tid = threadIdx.x, tile = PACK ? blockIdx.x / SP : blockIdx.x;
   const int c0 = tile * blockDim.x * CB + tid;
-#pragma unroll
-  for (int u = 0; u < CB; ++u) {  // a column past the end reads the thread's first
-    const int q = c0 + u * (int)blockDim.x < cols ? c0 + u * blockDim.x : min(c0, cols - 1);
-    const int a = q / C, c = q - a * C;
-    src[u] = reinterpret_cast<const P2 *>(in) + (b * A + a) * (long)N * C + c;
-    dst[u] = reinterpret_cast<P2 *>(out) + (b * A + a) * (long)nt * C + c;
-  }
+  const bool idle = c0 >= (PACK ? A * C : C);
+  const int a = PACK ? min(c0, A * C - 1) / C : blockIdx.y;
+  const int c = PACK ? min(c0, A * C - 1) - a * C : blockIdx.x * blockDim.x * CB + threadIdx.x;
+  const P2 *src = reinterpret_cast<const P2 *>(in) + (b * A + a) * (long)N * C + c;
   const C2<T> *eb = E + b * es + (long)axis * N * nt;
-  for (int j0 = (blockIdx.x - tile * SP) * JB; j0 < nt; j0 += SP * JB) {
+  P2 *dst = reinterpret_cast<P2 *>(out) + (b * A + a) * (long)nt * C + c;
+  int off[CB];  // a column past the end reads the thread's first
+#pragma unroll
+  for (int u = 0; u < CB; ++u) off[u] = !PACK && c + u * (int)blockDim.x < C ? u * blockDim.x : 0;
+  for (int j0 = PACK ? (blockIdx.x - tile * SP) * JB : 0; j0 < nt; j0 += PACK ? SP * JB : JB) {
     __syncthreads();
     for (int t = tid; t < N * JB; t += blockDim.x) {
       const int k = t / JB, j = j0 + t % JB;
@@ -631,8 +632,7 @@ k_idft_mid(const C2<T> *__restrict__ in, C2<T> *__restrict__ out, const C2<T> *_
       Es[t] = Q{e.x, e.x, -e.y, e.y};
     }
     __syncthreads();
-    if (c0 >= cols) continue;
-    const int nj = min(JB, nt - j0);
+    if (idle) continue;
     P2 acc[CB][JB];
 #pragma unroll
     for (int u = 0; u < CB; ++u)
@@ -645,7 +645,7 @@ k_idft_mid(const C2<T> *__restrict__ in, C2<T> *__restrict__ out, const C2<T> *_
       for (int q = 0; q < U; ++q)
 #pragma unroll
         for (int u = 0; u < CB; ++u)
-          if (k0 + q < N) nx[q][u] = src[u][(long)(k0 + q) * C];
+          if (k0 + q < N) nx[q][u] = src[(long)(k0 + q) * C + off[u]];
     };
     load(0);
     for (int k0 = 0; k0 < N; k0 += U) {
@@ -660,7 +660,7 @@ k_idft_mid(const C2<T> *__restrict__ in, C2<T> *__restrict__ out, const C2<T> *_
         if (k0 + q >= N) break;
 #pragma unroll
         for (int j = 0; j < JB; ++j) {
-          if (sizeof(T) == 8 && j >= nj) break;
+          if (sizeof(T) == 8 && j0 + j >= nt) break;
           const Q e = Es[(k0 + q) * JB + j];
 #pragma unroll
           for (int u = 0; u < CB; ++u) acc[u][j] = cmac(acc[u][j], v[q][u], e);
@@ -669,10 +669,10 @@ k_idft_mid(const C2<T> *__restrict__ in, C2<T> *__restrict__ out, const C2<T> *_
     }
 #pragma unroll
     for (int u = 0; u < CB; ++u)
-      if (u == 0 || c0 + u * (int)blockDim.x < cols)
+      if (u == 0 || off[u])
 #pragma unroll
         for (int j = 0; j < JB; ++j)
-          if (j < nj) dst[u][(long)(j0 + j) * C] = acc[u][j];
+          if (j0 + j < nt) dst[(long)(j0 + j) * C + off[u]] = acc[u][j];
   }
 }
 
@@ -820,10 +820,10 @@ static cudaError_t idft_grid(const Plan &p, int B, int nt, const double *org, in
     constexpr int CB = decltype(cb)::value;
     if constexpr (sizeof(T) == 4) {
       if (!few)
-        return wide == 4 ? k_idft_mid<T, 4, CB> : wide == 8 ? k_idft_mid<T, 8, CB>
-             : wide == 12 ? k_idft_mid<T, 12, CB> : k_idft_mid<T, 16, CB>;
+        return wide == 4 ? k_idft_mid<T, 4, CB, false> : wide == 8 ? k_idft_mid<T, 8, CB, false>
+             : wide == 12 ? k_idft_mid<T, 12, CB, false> : k_idft_mid<T, 16, CB, false>;
     }
-    return k_idft_mid<T, 4, 1>;
+    return k_idft_mid<T, 4, 1, true>;
   };
   auto midz = pick(std::integral_constant<int, 2>{}, fewz), midy = pick(std::integral_constant<int, 1>{}, fewy);
   const size_t smz = 2 * cs * (size_t)N * (fewz ? 4 : wide), smy = 2 * cs * (size_t)N * (fewy ? 4 : wide);
@@ -836,14 +836,12 @@ static cudaError_t idft_grid(const Plan &p, int B, int nt, const double *org, in
     return e;
   // FP64: CTAs of two warps, which end more evenly (64 volumes of 24^3, 11 points, z
   // stage: 139 us with four, 120 with two)
-  const int spz = fewz ? narrow : 1, spy = fewy ? narrow : 1, few_threads = sizeof(T) == 8 ? 64 : 128;
-  const int thz = fewz ? few_threads : 128, colz = fewz ? thz : 256;
-  midz<<<dim3((unsigned)((N2 + colz - 1) / colz * spz), 1, B), thz, smz, st>>>(
-      (const C2<T> *)w.Z, (C2<T> *)w.Y1, (const C2<T> *)w.E, N, nt, 1, (int)N2, 2, es, spz);
-  // (as many threads as columns of a row where the rows make enough CTAs)
-  const int thy = fewy ? few_threads : ty, coly = nt * N;
-  midy<<<dim3((unsigned)((coly + thy - 1) / thy * spy), 1, B), thy, smy, st>>>(
-      (const C2<T> *)w.Y1, (C2<T> *)w.Y2, (const C2<T> *)w.E, N, nt, nt, N, 1, es, spy);
+  const int thp = sizeof(T) == 8 ? 64 : 128;
+  auto packed = [&](long cols) { return dim3((unsigned)((cols + thp - 1) / thp * narrow), 1, B); };
+  midz<<<fewz ? packed(N2) : dim3((unsigned)((N2 + 255) / 256), 1, B), fewz ? thp : 128, smz, st>>>(
+      (const C2<T> *)w.Z, (C2<T> *)w.Y1, (const C2<T> *)w.E, N, nt, 1, (int)N2, 2, es, narrow);
+  midy<<<fewy ? packed((long)nt * N) : dim3((N + ty - 1) / ty, nt, B), fewy ? thp : ty, smy, st>>>(
+      (const C2<T> *)w.Y1, (C2<T> *)w.Y2, (const C2<T> *)w.E, N, nt, nt, N, 1, es, narrow);
   k_idft_x<T><<<dim3((rows + 7) / 8, B), 256, smx, st>>>(
       (const C2<T> *)w.Y2, (T *)w.CC, (const C2<T> *)w.E, N, nt, rows, T(1.0 / ((double)N2 * N)), es);
   k_cc_argmax<T><<<B, 256, 0, st>>>((const T *)w.CC, nt, org, j0, den, edge, flag_mode, R, t_out,
