@@ -168,7 +168,12 @@ constexpr int ANALYZE_THREADS = 192;
 // CTAs per SM) or spill under a four-CTA bound, and both measure slower
 constexpr int GATHER_BATCH = 2;
 
-struct TexPair { TexArgs of[2]; };
+// The views of a launch's one or two batches, in one array: each 2 KB of parameters is
+// up to 2 us of a small launch.
+struct TexPair {
+  cudaTextureObject_t t[TEX_MAX];
+  int vpt[2], first[2];
+};
 template <typename T, int G, bool TEX>
 __global__ void __launch_bounds__(ANALYZE_THREADS)
 k_analyze2(const float *__restrict__ vols, int B0, const float *__restrict__ vols2, int N, int S, int L,
@@ -215,8 +220,8 @@ k_analyze2(const float *__restrict__ vols, int B0, const float *__restrict__ vol
   cudaTextureObject_t tob = 0;
   float yoff = 0.f;  // first row of this volume in its texture view
   if (TEX) {
-    const int vpt = ta.of[second].vpt, run = (int)b / vpt;
-    tob = ta.of[second].t[run];
+    const int vpt = ta.vpt[second], run = (int)b / vpt;
+    tob = ta.t[ta.first[second] + run];
     yoff = (float)((b - (long)run * vpt) * NN);
   }
   // trilinear combination of the two gathered planes (components: x (i, j+1),
@@ -553,8 +558,10 @@ static AnalyzeShape analyze_shape(const Plan &p, long volumes) {
   }
   G = G >= 8 ? 8 : G >= 4 ? 4 : G >= 2 ? 2 : 1;
   while (G > 1 && (p.S % G != 0 || analyze2_smem<T>(p, G) > 100 * 1024)) G >>= 1;
-  // three CTAs on 164 KB, or two where the box is large
-  const bool cap = sizeof(T) == 4 && G == 1 && p.N >= 88 && cost(1) <= 164 * 1024 / (p.N > 128 ? 2 : 3);
+  // three CTAs on 164 KB, or two where the box is large (plans whose four CTAs fit 132
+  // KB are left to the driver: 64 of 160^3, L_J = 30: 119 us, 124 with the limit)
+  const bool cap = sizeof(T) == 4 && G == 1 && p.N >= 88 && 4 * cost(1) > 132 * 1024 &&
+                   cost(1) <= 164 * 1024 / (p.N > 128 ? 2 : 3);
   return {G, cap ? 71 : -1};
 }
 
@@ -572,9 +579,20 @@ cudaError_t launch_analyze(const Plan &p, const float *vols, int B, T *coef, cud
     size_t smem = analyze2_smem<T>(p, G);
     if (smem <= 200 * 1024 && (long)B + B2 <= 65535) {
       std::lock_guard<std::mutex> lock(p.tex_mu);
+      TexArgs views, views2;
+      const bool tex = texture_views(p, vols, B, st, views);
+      const bool tex2 = B2 > 0 ? texture_views(p, vols2, B2, st, views2) : tex;
       TexPair tp;
-      const bool tex = texture_views(p, vols, B, st, tp.of[0]);
-      const bool tex2 = B2 > 0 ? texture_views(p, vols2, B2, st, tp.of[1]) : tex;
+      auto load = [&](const TexArgs &v, int n, int which, int first) {
+        const int runs = (n + v.vpt - 1) / v.vpt;
+        if (first + runs > TEX_MAX) return -1;
+        std::copy_n(v.t, runs, tp.t + first);
+        tp.vpt[which] = v.vpt;
+        tp.first[which] = first;
+        return first + runs;
+      };
+      const int held = tex ? load(views, B, 0, 0) : 0;
+      const bool together = tex == tex2 && (!tex || B2 == 0 || load(views2, B2, 1, held) > 0);
       auto pick = [&](auto tag) {
         constexpr bool X = decltype(tag)::value;
         return G == 8 ? k_analyze2<T, 8, X> : G == 4 ? k_analyze2<T, 4, X>
@@ -598,10 +616,10 @@ cudaError_t launch_analyze(const Plan &p, const float *vols, int B, T *coef, cud
             p.Mq, (const T *)p.ptab_leg, p.leg_lm, (const T *)p.ring, o, coef2, tp);
         return cudaGetLastError();
       };
-      if (tex == tex2) return run(tex, vols, B, coef, B2);
+      if (together) return run(tex, vols, B, coef, B2);
       const cudaError_t e = run(tex, vols, B, coef, 0);
       if (e != cudaSuccess) return e;
-      tp.of[0] = tp.of[1];
+      if (tex2) load(views2, B2, 0, 0);
       return run(tex2, vols2, B2, coef2, 0);
     }
   }
