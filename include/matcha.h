@@ -307,7 +307,8 @@ matcha_status matcha_align_host(matcha_plan plan, const float *particles, const 
 typedef struct {
   int analyze_shells;
   float analyze_ms[4];     /* candidates 1, 2, 4, 8 shells per CTA */
-  int tc_ctas_per_sm;      /* 0 when the plan's contraction runs on the CUDA cores */
+  int tc_ctas_per_sm;      /* 0 when the plan's contraction runs on the CUDA cores, or the
+                              batch in blocks of particles against its one template */
   float tc_ms[2];          /* candidates 1, 2 CTAs per SM */
   int soft_kernel;         /* 0 when only one SOFFT kernel serves the plan */
   float soft_ms[3];        /* candidates 1 (chunked), 2 (warp per slice), 3 (register-tiled) */

@@ -700,21 +700,17 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
 
 }  // namespace
 
-cudaError_t launch_correlate_tc(const Plan &p, const float *f, const float *h, int B, int hstride,
-                                float *c, cudaStream_t st) {
-  if (B == 0) return cudaSuccess;
-  const int bf16 = p.tc == 2;
-  const TcGeom g = tc_geom(p.S, p.LJ, bf16 ? 2 : 4);
-  if (!correlate_tc_fits(p.S, p.LJ, bf16 ? 2 : 4) || p.S > 128) return cudaErrorInvalidConfiguration;
+// Particles per block: their passes share one staging of B, worth about 2.5 particles,
+// but the blocks have to fill the SMs (at most 16: those in flight then write about 64
+// MB, so that the degrees of an output line meet in L2).  An item of k_correlate_tc, two
+// on an SM, takes about as long as 4.2 particles of a pass.  768 particles, 32 shells,
+// L_J = 48, TF32: 387 us with 8, 351 with 16; 17 and 64 particles, 24 shells, L_J = 33:
+// 14 and 31 us with k_correlate_tc, 20 and 34 in blocks of two, 17 and 23 in blocks of
+// four and eight.
+// 0: k_correlate_tc.
+int correlate_tc_block(const Plan &p, int B, int hstride) {
   const int nsm = p.sms;
-  const int PM = hstride ? 0 : tc_shared_stack(g, p.S, p.LJ);
-  // Particles per block: their passes share one staging of B, worth about 2.5 particles,
-  // but the blocks have to fill the SMs (at most 16: those in flight then write about 64
-  // MB, so that the degrees of an output line meet in L2).  An item of k_correlate_tc, two
-  // on an SM, takes about as long as 4.2 particles of a pass.  768 particles, 32 shells,
-  // L_J = 48, TF32: 387 us with 8, 351 with 16; 17 and 64 particles, 24 shells, L_J = 33:
-  // 14 and 31 us with k_correlate_tc, 20 and 34 in blocks of two, 17 and 23 in blocks of
-  // four and eight.
+  const int PM = hstride ? 0 : tc_shared_stack(tc_geom(p.S, p.LJ, p.tc == 2 ? 2 : 4), p.S, p.LJ);
   const int pairs = p.LJ / 2 + 1;
   const long items = (long)B * pairs;
   int PB = 0;
@@ -724,9 +720,20 @@ cudaError_t launch_correlate_tc(const Plan &p, const float *f, const float *h, i
     const double t = (units + nsm - 1) / nsm * (2.5 + q);
     if (t < best) { best = t; PB = q; }
   }
-  const bool shared = PB && items > 2L * nsm && best <= 4.2 * ((items + 2L * nsm - 1) / (2L * nsm));
-  if (shared) {
-    const long units = (long)((B + PB - 1) / PB) * pairs;
+  return items > 2L * nsm && best <= 4.2 * ((items + 2L * nsm - 1) / (2L * nsm)) ? PB : 0;
+}
+
+cudaError_t launch_correlate_tc(const Plan &p, const float *f, const float *h, int B, int hstride,
+                                float *c, cudaStream_t st) {
+  if (B == 0) return cudaSuccess;
+  const int bf16 = p.tc == 2;
+  const TcGeom g = tc_geom(p.S, p.LJ, bf16 ? 2 : 4);
+  if (!correlate_tc_fits(p.S, p.LJ, bf16 ? 2 : 4) || p.S > 128) return cudaErrorInvalidConfiguration;
+  const int nsm = p.sms, PB = correlate_tc_block(p, B, hstride);
+  const long items = (long)B * (p.LJ / 2 + 1);
+  if (PB) {
+    const int PM = tc_shared_stack(g, p.S, p.LJ);
+    const long units = (long)((B + PB - 1) / PB) * (p.LJ / 2 + 1);
     const int smem1 = (int)tc_shared(g, p.LJ, PM).smem;
     const long limit = p.wait_limit >= 0 ? p.wait_limit : TC_WAIT_LIMIT;
     auto kern = bf16 ? k_correlate_tc_shared<1> : k_correlate_tc_shared<0>;

@@ -195,6 +195,7 @@ cudaError_t launch_template_grad(const Plan &p, const T *f, const T *c, int B, i
 cudaError_t launch_correlate_tc(const Plan &p, const float *f, const float *h, int B, int hstride,
                                 float *c, cudaStream_t st);
 bool correlate_tc_fits(int S, int L, int bytes);
+int correlate_tc_block(const Plan &p, int B, int hstride);  // particles per block, 0: single ones
 bool backward_fits(const Plan &p);  // the template-gradient kernel's shared memory fits
 int newton_slots(const Plan &p);                  // sub-slots of a particle's sums
 size_t newton_smem(const Plan &p);                // of one CTA per particle

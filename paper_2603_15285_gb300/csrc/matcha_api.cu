@@ -744,7 +744,10 @@ matcha_status matcha_plan_autotune(matcha_plan plan, const float *particles, con
   }
   p->tune_shells = bestG;
   rep->analyze_shells = bestG;
-  if (err == cudaSuccess && p->tc) {
+  if (p->tc && correlate_tc_block(*p, B, tstride)) {  // blocks of particles: one CTA per SM
+    rep->tc_ms[0] = rep->tc_ms[1] = -1.0f;
+    p->tune_tc_ctas = 0;
+  } else if (err == cudaSuccess && p->tc) {
     const int Bt = tstride ? B : 1;
     err = launch_analyze<float>(*p, particles, B, (float *)w.f, st);
     if (err == cudaSuccess) err = launch_analyze<float>(*p, templates, Bt, (float *)w.h, st);
