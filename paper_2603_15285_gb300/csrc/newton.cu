@@ -837,29 +837,26 @@ cudaError_t launch_newton(const Plan &p, const T *c, int B, const int *n_cand, d
   if (B == 0) return cudaSuccess;
   cudaError_t e;
   if (launch_newton_spread<T>(p, c, B, std::max(B, batch), n_cand, euler, score, cflags, work, st, &e)) return e;
-  NewtonArgs A;
-  A.LJ = p.LJ; A.nlev = p.nlev; A.M = p.M; A.P = p.P;
-  A.cpw = newton_cpw(p.P);
-  A.nslots = newton_slots(p, sizeof(T));
-  if (A.nslots == 0) return cudaErrorInvalidConfiguration;
-  for (int i = 0; i < MATCHA_MAX_LEVELS; ++i) A.Ls[i] = i < p.nlev ? p.Ls[i] : 0;
-  A.tol = p.step_tol;
-  A.acc_tol = p.accept_tol;
-  A.grad = p.refine;
-  A.nc = p.nc;
-  size_t smem = newton_smem_bytes(p, sizeof(T), A.nslots);
-  if constexpr (sizeof(T) == 4) {
-    if (newton_rescaled(p)) {
-      if ((e = allow_smem(k_newton<T, true>, smem)) != cudaSuccess) return e;
-      k_newton<T, true><<<B, NEWTON_THREADS, smem, st>>>(c, (const T *)p.rcoef, (const T *)p.seedK,
-                                                         A, n_cand, euler, score, cflags, work);
-      return cudaGetLastError();
-    }
+  if constexpr (sizeof(T) == 8) {
+    return cudaErrorInvalidConfiguration;  // FP64 plans have a spread shape each
+  } else {
+    NewtonArgs A;
+    A.LJ = p.LJ; A.nlev = p.nlev; A.M = p.M; A.P = p.P;
+    A.cpw = newton_cpw(p.P);
+    A.nslots = newton_slots(p, sizeof(T));
+    if (A.nslots == 0) return cudaErrorInvalidConfiguration;
+    for (int i = 0; i < MATCHA_MAX_LEVELS; ++i) A.Ls[i] = i < p.nlev ? p.Ls[i] : 0;
+    A.tol = p.step_tol;
+    A.acc_tol = p.accept_tol;
+    A.grad = p.refine;
+    A.nc = p.nc;
+    const size_t smem = newton_smem_bytes(p, sizeof(T), A.nslots);
+    auto kern = newton_rescaled(p) ? k_newton<T, true> : k_newton<T, false>;
+    if ((e = allow_smem(kern, smem)) != cudaSuccess) return e;
+    kern<<<B, NEWTON_THREADS, smem, st>>>(c, (const T *)p.rcoef, (const T *)p.seedK, A, n_cand, euler, score,
+                                          cflags, work);
+    return cudaGetLastError();
   }
-  if ((e = allow_smem(k_newton<T, false>, smem)) != cudaSuccess) return e;
-  k_newton<T, false><<<B, NEWTON_THREADS, smem, st>>>(c, (const T *)p.rcoef, (const T *)p.seedK,
-                                                      A, n_cand, euler, score, cflags, work);
-  return cudaGetLastError();
 }
 
 template <typename T>
@@ -906,26 +903,22 @@ cudaError_t launch_objective(const Plan &p, const T *c, int B, int L, int Q, con
   if (B == 0 || Q == 0) return cudaSuccess;
   cudaError_t e;
   if (launch_objective_spread<T>(p, c, B, L, Q, pts, out, st, &e)) return e;
-  NewtonArgs A;
-  A.LJ = p.LJ; A.nlev = p.nlev; A.M = p.M; A.P = p.P;
-  A.cpw = newton_cpw(p.P);
-  A.nslots = newton_slots(p, sizeof(T));
-  if (A.nslots == 0) return cudaErrorInvalidConfiguration;
-  for (int i = 0; i < MATCHA_MAX_LEVELS; ++i) A.Ls[i] = i < p.nlev ? p.Ls[i] : 0;
-  A.tol = p.step_tol; A.acc_tol = p.accept_tol; A.grad = p.refine; A.nc = p.nc;
-  size_t smem = newton_smem_bytes(p, sizeof(T), A.nslots);
-  if constexpr (sizeof(T) == 4) {
-    if (newton_rescaled(p)) {
-      if ((e = allow_smem(k_objective<T, true>, smem)) != cudaSuccess) return e;
-      k_objective<T, true><<<B, NEWTON_THREADS, smem, st>>>(c, (const T *)p.rcoef,
-                                                            (const T *)p.seedK, A, L, Q, pts, out);
-      return cudaGetLastError();
-    }
+  if constexpr (sizeof(T) == 8) {
+    return cudaErrorInvalidConfiguration;  // as launch_newton
+  } else {
+    NewtonArgs A;
+    A.LJ = p.LJ; A.nlev = p.nlev; A.M = p.M; A.P = p.P;
+    A.cpw = newton_cpw(p.P);
+    A.nslots = newton_slots(p, sizeof(T));
+    if (A.nslots == 0) return cudaErrorInvalidConfiguration;
+    for (int i = 0; i < MATCHA_MAX_LEVELS; ++i) A.Ls[i] = i < p.nlev ? p.Ls[i] : 0;
+    A.tol = p.step_tol; A.acc_tol = p.accept_tol; A.grad = p.refine; A.nc = p.nc;
+    const size_t smem = newton_smem_bytes(p, sizeof(T), A.nslots);
+    auto kern = newton_rescaled(p) ? k_objective<T, true> : k_objective<T, false>;
+    if ((e = allow_smem(kern, smem)) != cudaSuccess) return e;
+    kern<<<B, NEWTON_THREADS, smem, st>>>(c, (const T *)p.rcoef, (const T *)p.seedK, A, L, Q, pts, out);
+    return cudaGetLastError();
   }
-  if ((e = allow_smem(k_objective<T, false>, smem)) != cudaSuccess) return e;
-  k_objective<T, false><<<B, NEWTON_THREADS, smem, st>>>(c, (const T *)p.rcoef, (const T *)p.seedK,
-                                                         A, L, Q, pts, out);
-  return cudaGetLastError();
 }
 template cudaError_t launch_objective<float>(const Plan &, const float *, int, int, int,
                                              const double *, double *, cudaStream_t);

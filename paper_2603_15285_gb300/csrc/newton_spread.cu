@@ -350,8 +350,8 @@ __device__ __forceinline__ void particle_sync(const SpreadArgs &A) {
 // Evaluates C (and grad, Hessian when FULL) at pts[p] for the candidates with
 // need[p] != 0; results in res[p][0..9] (FP64) of every CTA of the particle.
 // Called by all of them.
-// SPLIT: W workers per chain group and z in shared memory; else one, which adds
-// its groups' images to accumulators in registers.
+// SPLIT (32-bit plans): W workers per chain group and z in shared memory; else (FP64)
+// one, which adds its groups' images to accumulators in registers.
 template <typename T, bool FULL, bool RS, bool SPLIT>
 __device__ __forceinline__ void evaluate(const SpreadArgs &A, int L, const T *__restrict__ cb,
                                          const T *__restrict__ rcoef, const T *__restrict__ gdesc,
@@ -803,7 +803,8 @@ size_t spread_smem(const Plan &p, size_t tsize, SpreadArgs &A) {
 
 // The shape for B particles, or false where one CTA per particle is as fast.
 //
-// FP64: one worker per chain group.  An SM's FP64 pipe is full from about four of
+// FP64: one worker per chain group, and a shape for every plan (one chain group per CTA
+// fits wherever the plan's refinement does).  An SM's FP64 pipe is full from about four of
 // these warps on (40 particles to L = 32: 8.1 ms at eight warps per SM, 4.5 at
 // four, 4.4 at two), so a wave of resident CTAs costs max(4, its warps); one CTA
 // per particle, 9.0 ms, is never faster.
@@ -911,16 +912,16 @@ int newton_schedule(const Plan &p, std::vector<int4> &out) {
   return rounds;
 }
 
-// False when one CTA per particle is expected to be as fast.
+// False when one CTA per particle is expected to be as fast (32-bit plans).
 template <typename T>
 bool launch_newton_spread(const Plan &p, const T *c, int B, int batch, const int *n_cand, double *euler,
                           double *score, int *cflags, long long *work, cudaStream_t st, cudaError_t *e) {
   SpreadArgs A;
   size_t smem;
   if (!spread_shape(p, sizeof(T), batch, A, &smem)) return false;
-  auto kern = A.W > 1 ? k_newton_spread<T, false, true> : k_newton_spread<T, false, false>;
+  auto kern = k_newton_spread<T, false, sizeof(T) == 4>;
   if constexpr (sizeof(T) == 4)
-    if (newton_rescaled(p)) kern = A.W > 1 ? k_newton_spread<T, true, true> : k_newton_spread<T, true, false>;
+    if (newton_rescaled(p)) kern = k_newton_spread<T, true, true>;
   *e = launch_clusters(kern, B, A, smem, st, c, (const T *)p.rcoef, (const T *)p.gdesc, A, n_cand, euler,
                        score, cflags, work);
   return true;
@@ -936,9 +937,9 @@ bool launch_objective_spread(const Plan &p, const T *c, int B, int L, int Q, con
   SpreadArgs A;
   size_t smem;
   if (!spread_shape(p, sizeof(T), B, A, &smem)) return false;
-  auto kern = A.W > 1 ? k_objective_spread<T, false, true> : k_objective_spread<T, false, false>;
+  auto kern = k_objective_spread<T, false, sizeof(T) == 4>;
   if constexpr (sizeof(T) == 4)
-    if (newton_rescaled(p)) kern = A.W > 1 ? k_objective_spread<T, true, true> : k_objective_spread<T, true, false>;
+    if (newton_rescaled(p)) kern = k_objective_spread<T, true, true>;
   *e = launch_clusters(kern, B, A, smem, st, c, (const T *)p.rcoef, (const T *)p.gdesc, A, L, Q, pts, out);
   return true;
 }
