@@ -219,7 +219,7 @@ bool soft_tile_ok(const Plan &p);        // the register-tiled SOFFT kernel serv
 // Translation search (translate.cu): volume poses, the box FFT, the cross
 // spectrum and the windowed inverse DFT of the correlation.
 cudaError_t launch_pose_volumes(int N, const float *vol, int B, long vol_stride, const double *R,
-                                const double *shift, bool fp64, float *out, cudaStream_t st);
+                                const double *shift, bool fp64, int sms, float *out, cudaStream_t st);
 struct ShiftWs {
   void *Z;        // complex [B][N^3] (plan precision): spectra, then the cross spectrum
   void *Y1, *Y2;  // complex [B][nt][N^2], [B][nt][nt][N]

@@ -78,8 +78,12 @@ extern "C" matcha_status matcha_transform_volumes(int N, const float *vols, int 
   if (B > 65535) return MATCHA_ERR_UNSUPPORTED;
   if (precision < MATCHA_FP64 || precision > MATCHA_BF16) return MATCHA_ERR_INVALID_ARG;
   const long vox = (long)N * N * N;
-  cudaError_t e = launch_pose_volumes(N, vols, B, vol_stride ? vox : 0, R, shift,
-                                      precision == MATCHA_FP64, out, (cudaStream_t)stream);
+  int dev = 0, sms = 1;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e == cudaSuccess)
+    e = launch_pose_volumes(N, vols, B, vol_stride ? vox : 0, R, shift, precision == MATCHA_FP64, sms, out,
+                            (cudaStream_t)stream);
   if (e != cudaSuccess) return cuda_fail(e, "matcha_transform_volumes");
   return MATCHA_OK;
 }
@@ -156,7 +160,7 @@ extern "C" matcha_status matcha_align6d(matcha_plan plan, const float *particles
     const float *tr = templates;
     int ts = tstride;
     if (r > 0) {
-      cudaError_t e = launch_pose_volumes(p.N, templates, B, tstride ? vox : 0, nullptr, tau, fp64,
+      cudaError_t e = launch_pose_volumes(p.N, templates, B, tstride ? vox : 0, nullptr, tau, fp64, p.sms,
                                           w.shifted, st);
       if (e != cudaSuccess) return cuda_fail(e, "matcha_align6d: shift");
       tr = w.shifted;
@@ -166,7 +170,7 @@ extern "C" matcha_status matcha_align6d(matcha_plan plan, const float *particles
                                    flags, w.align_ws, w.align_bytes, stream);
     if (s != MATCHA_OK) return s;
     // translation search of the rotated template u = g o h
-    cudaError_t e = launch_pose_volumes(p.N, templates, B, tstride ? vox : 0, R, nullptr, fp64,
+    cudaError_t e = launch_pose_volumes(p.N, templates, B, tstride ? vox : 0, R, nullptr, fp64, p.sms,
                                         w.rotated, st);
     if (e != cudaSuccess) return cuda_fail(e, "matcha_align6d: rotate");
     e = fp64 ? launch_shift_search<double>(p, particles, w.rotated, B, max_shift, upsample, R, w.sw,

@@ -712,7 +712,7 @@ cudaError_t launch_soft_grid(const Plan &p, const T *c, int B, const int *P_per,
   // batch still fills two CTAs on every SM and two fit an SM
   const int tiles = (round_up(p.ns, Tile<T>::I) / Tile<T>::I) * (round_up(p.ns, Tile<T>::J) / Tile<T>::J);
   int KS = std::max(1, 256 / tiles);
-  while (KS > 1 && ((long)B * p.ns < 304L * KS || slab_rows<T>(p, KS) < round_up(p.ns, Tile<T>::I))) --KS;
+  while (KS > 1 && ((long)B * p.ns < 2L * p.sms * KS || slab_rows<T>(p, KS) < round_up(p.ns, Tile<T>::I))) --KS;
   const int IC = (int)slab_rows<T>(p, KS);
   if (IC == 0) return cudaErrorInvalidConfiguration;
   const size_t smem = sizeof(T) * slab_reals<T>(p.L0, p.ns, KS, IC);
@@ -730,7 +730,7 @@ cudaError_t launch_soft_grid(const Plan &p, const T *c, int B, const int *P_per,
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeClusterDimension;
   at[0].val.clusterDim.x = 8;
-  while (at[0].val.clusterDim.x > 1 && (long)B * at[0].val.clusterDim.x > 304) at[0].val.clusterDim.x /= 2;
+  while (at[0].val.clusterDim.x > 1 && (long)B * at[0].val.clusterDim.x > 2L * p.sms) at[0].val.clusterDim.x /= 2;
   at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
   cfg.gridDim = dim3(at[0].val.clusterDim.x * B);
   cfg.blockDim = dim3(PEAK_THREADS);

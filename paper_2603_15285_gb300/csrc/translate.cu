@@ -173,13 +173,13 @@ k_pose_volume64(int N, const float *__restrict__ vol, long vstride, const double
 }
 
 cudaError_t launch_pose_volumes(int N, const float *vol, int B, long vol_stride, const double *R,
-                                const double *shift, bool fp64, float *out, cudaStream_t st) {
+                                const double *shift, bool fp64, int sms, float *out, cudaStream_t st) {
   if (B <= 0) return cudaSuccess;
   if (fp64) {
     // four voxels per thread where that leaves at most a thirtieth of the lanes idle and
-    // makes six CTAs on each of 152 SMs, whose work then ends evenly; else one
+    // makes six CTAs on each SM, whose work then ends evenly; else one
     const int planes = (N * N + POSE_THREADS - 1) / POSE_THREADS, quads = (N + 3) / 4;
-    if (30L * N * N * N >= 29L * planes * POSE_THREADS * quads * 4 && (long)planes * quads * B >= 912)
+    if (30L * N * N * N >= 29L * planes * POSE_THREADS * quads * 4 && (long)planes * quads * B >= 6L * sms)
       k_pose_volume64<4><<<dim3(planes, quads, B), POSE_THREADS, 0, st>>>(N, vol, vol_stride, R, shift, out);
     else
       k_pose_volume64<1><<<dim3((N * N * N + POSE_THREADS - 1) / POSE_THREADS, 1, B), POSE_THREADS, 0, st>>>(
@@ -192,8 +192,8 @@ cudaError_t launch_pose_volumes(int N, const float *vol, int B, long vol_stride,
     const dim3 grid((unsigned)(nbx * nby), (unsigned)((N + POSE_Z * ST - 1) / (POSE_Z * ST)), B);
     k_pose_volume<ST><<<grid, POSE_THREADS, 0, st>>>(N, nbx, vol, vol_stride, R, shift, out);
   };
-  // eight voxels per thread where that still makes four CTAs on each of 152 SMs
-  if ((long)nbx * nby * ((N + 31) / 32) * B >= 608) run(std::integral_constant<int, 8>{});
+  // eight voxels per thread where that still makes four CTAs on each SM
+  if ((long)nbx * nby * ((N + 31) / 32) * B >= 4L * sms) run(std::integral_constant<int, 8>{});
   else run(std::integral_constant<int, 2>{});
   return cudaGetLastError();
 }
