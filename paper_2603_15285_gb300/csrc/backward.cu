@@ -662,12 +662,14 @@ cudaError_t launch_template_grad(const Plan &p, const T *f, const T *c, int B, i
   T *Xo = tstride ? coef_grad : X;
   point<<<B, BWD_THREADS, ps, st>>>(c, 4L * p.nc, (const T *)p.rcoef, (const T *)p.seedK, p.LJ, euler,
                                     shift, flags);
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
   k_bwd_coef<T><<<dim3(B, (p.S + Sc - 1) / Sc), BWD_THREADS, smem, st>>>(
       f, p.S, Sc, p.LJ, p.wrad, (const T *)p.rcoef, (const T *)p.seedK, euler, shift, weight, Xo);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   const int ntmpl = tstride ? B : 1;
   if (!tstride)
     k_bwd_reduce<T><<<(int)((per + RED_X - 1) / RED_X), dim3(RED_X, RED_Y), 0, st>>>(X, B, per, coef_grad);
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
   if (vox_grad) {
     const long nv = (long)p.N * p.N * p.N * ntmpl;
     e = cudaMemsetAsync(vox_grad, 0, sizeof(double) * nv, st);

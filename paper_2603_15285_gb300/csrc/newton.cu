@@ -873,6 +873,8 @@ cudaError_t launch_newton_queue(const Plan &p, const T *c, int B, const int *n_c
   A.tol = p.step_tol; A.acc_tol = p.accept_tol; A.grad = p.refine; A.nc = p.nc;
   const size_t smem = newton_smem_bytes(p, sizeof(T), A.nslots);
   k_cost_order<<<1, 1024, 0, st>>>(n_cand, B, p.P, order, ticket);
+  cudaError_t launched = cudaGetLastError();
+  if (launched != cudaSuccess) return launched;
   int dev = 0, sms = 0, per_sm = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);

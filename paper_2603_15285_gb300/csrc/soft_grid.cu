@@ -721,6 +721,7 @@ cudaError_t launch_soft_grid(const Plan &p, const T *c, int B, const int *P_per,
   (cvec ? k_soft_beta<T, true> : k_soft_beta<T, false>)
       <<<dim3((ng + BETA_GROUPS - 1) / BETA_GROUPS, (B + BETA_NB - 1) / BETA_NB), 128, 0, st>>>(
           c, p.nc, p.LJ, p.L0, p.ns, B, (const T *)p.soft_dT, grid);
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
   k_soft_slab<T><<<dim3((p.ns + KS - 1) / KS, B), 256, smem, st>>>(p.L0, p.ns, KS, IC,
                                                                    (const T *)p.soft_tw, grid, vec);
   e = cudaGetLastError();

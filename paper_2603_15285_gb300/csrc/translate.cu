@@ -805,6 +805,8 @@ static cudaError_t idft_grid(const Plan &p, int B, int nt, const double *org, in
   const int nb = org ? B : 1;
   const long es = org ? 3L * N * nt : 0;
   k_idft_factors<T><<<3 * nb * ((N * nt + 255) / 256), 256, 0, st>>>((C2<T> *)w.E, N, nt, org, j0, den);
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
   // z stage: X[b][kz][ky kx] -> Y1[b][tz][ky kx], then y stage: Y1[b][tz][ky][kx]
   // -> Y2[b][tz][ty][kx].  FP32: the grid points per pass over a column are the fewest
   // passes of at most 16, rounded up to 4, with two columns per thread in the z stage,
@@ -830,7 +832,6 @@ static cudaError_t idft_grid(const Plan &p, int B, int nt, const double *org, in
   // x stage: Y2[b][tz ty][kx] -> CC[b][tz ty][tx]
   const int rows = nt * nt;
   const size_t smx = cs * (8 * (size_t)N + (size_t)N * nt);
-  cudaError_t e;
   if ((e = allow_smem(midz, smz)) != cudaSuccess || (e = allow_smem(midy, smy)) != cudaSuccess ||
       (e = allow_smem(k_idft_x<T>, smx)) != cudaSuccess)
     return e;
@@ -840,10 +841,13 @@ static cudaError_t idft_grid(const Plan &p, int B, int nt, const double *org, in
   auto packed = [&](long cols) { return dim3((unsigned)((cols + thp - 1) / thp * narrow), 1, B); };
   midz<<<fewz ? packed(N2) : dim3((unsigned)((N2 + 255) / 256), 1, B), fewz ? thp : 128, smz, st>>>(
       (const C2<T> *)w.Z, (C2<T> *)w.Y1, (const C2<T> *)w.E, N, nt, 1, (int)N2, 2, es, narrow);
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
   midy<<<fewy ? packed((long)nt * N) : dim3((N + ty - 1) / ty, nt, B), fewy ? thp : ty, smy, st>>>(
       (const C2<T> *)w.Y1, (C2<T> *)w.Y2, (const C2<T> *)w.E, N, nt, nt, N, 1, es, narrow);
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
   k_idft_x<T><<<dim3((rows + 7) / 8, B), 256, smx, st>>>(
       (const C2<T> *)w.Y2, (T *)w.CC, (const C2<T> *)w.E, N, nt, rows, T(1.0 / ((double)N2 * N)), es);
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
   k_cc_argmax<T><<<B, 256, 0, st>>>((const T *)w.CC, nt, org, j0, den, edge, flag_mode, R, t_out,
                                     tau_out, cc_out, flags);
   return cudaGetLastError();
@@ -873,6 +877,7 @@ cudaError_t launch_shift_search(const Plan &p, const float *f, const float *u, i
     // registers kept other planes off the SM, 49 us with 256 threads, 24 with 64)
     const int threads = sizeof(T) == 8 ? std::min(256, std::max(64, (N * N / 4 + 31) / 32 * 32)) : 256;
     k_fft_plane<T><<<dim3(N, B), threads, plane, st>>>(Z, f, u, fd, tw);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
   } else {
     // rows, then columns (at least 16, so their rows stay coalesced), about 4096
     // elements per CTA; fewer where they and the twiddles exceed shared memory (FP64
@@ -884,8 +889,10 @@ cudaError_t launch_shift_search(const Plan &p, const float *f, const float *u, i
     const size_t sm0 = lines(NB0), sm1 = lines(NB);
     if ((e = allow_smem(k_fft_axis<T>, sm0 > sm1 ? sm0 : sm1)) != cudaSuccess) return e;
     k_fft_axis<T><<<dim3((unsigned)((N2 + NB0 - 1) / NB0), B), 256, sm0, st>>>(Z, f, u, 0, fd, tw, NB0);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
     k_fft_axis<T><<<dim3((unsigned)(N * ((N + NB - 1) / NB)), B), 256, sm1, st>>>(Z, nullptr, nullptr, 1,
                                                                                fd, tw, NB);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   // columns of the z transform per CTA: 128-byte rows while four buffers of them
   // leave two CTAs on an SM
