@@ -298,7 +298,8 @@ matcha_status matcha_align_host(matcha_plan plan, const float *particles, const 
  * 32-bit plans whose grid fits it the SOFFT search kernel (1: the chunked
  * kernels, 2: one warp per beta slice, 3: the register-tiled chunked kernel,
  * the built-in choice where it applies), and the refinement schedule of
- * matcha_align (1: one CTA per particle, 2: persistent CTAs on a cost-sorted
+ * matcha_align (1: a launch in index order, a particle on one CTA or spread
+ * over several while SMs are idle, 2: persistent CTAs on a cost-sorted
  * queue, longest processing time first).  P_per_dev (nullable) gives the
  * per-particle candidate counts as for matcha_align.  Uses the matcha_align workspace for
  * its scratch; synchronises `stream` (not graph-capturable: tune first, then
@@ -312,9 +313,9 @@ typedef struct {
   float tc_ms[2];          /* candidates 1, 2 CTAs per SM */
   int soft_kernel;         /* 0 when only one SOFFT kernel serves the plan */
   float soft_ms[3];        /* candidates 1 (chunked), 2 (warp per slice), 3 (register-tiled) */
-  int newton_sched;        /* matcha_align's refinement: 1 a CTA per particle in index
-                              order, 2 persistent CTAs pulling particles from a queue
-                              sorted by decreasing candidate count */
+  int newton_sched;        /* matcha_align's refinement: 1 a launch in index order (a CTA
+                              or a cluster per particle), 2 persistent CTAs pulling
+                              particles from a queue sorted by decreasing candidate count */
   float newton_ms[2];
 } matcha_tune_report;
 matcha_status matcha_plan_autotune(matcha_plan plan, const float *particles_dev,

@@ -49,7 +49,7 @@ struct Plan {
   int tune_tc_ctas = 0;  // tensor-core contraction CTAs per SM (1, 2)
   int tune_soft = 0;     // SOFFT search kernel: 1 the chunked kernels, 2 warp per slice,
                          // 3 register-tiled
-  int tune_newton = 0;   // refinement schedule: 1 a CTA per particle, 2 persistent cost-sorted queue
+  int tune_newton = 0;   // refinement schedule: 1 in index order, 2 persistent cost-sorted queue
   long wait_limit = -1;  // mbarrier polls before a wait gives up (-1: the built-in limit)
   int nt, np, nlm, npairs, npairs0, ns;
   int ngroups;  // partner groups of the correlation layout, (L_J+1)(L_J+2)/2
@@ -201,7 +201,7 @@ int newton_slots(const Plan &p);                  // sub-slots of a particle's s
 size_t newton_smem(const Plan &p);                // of one CTA per particle
 bool newton_rescaled(const Plan &p);              // the rescaled 32-bit recurrence runs
 int newton_schedule(const Plan &p, std::vector<int4> &out);  // returns the rounds
-template <typename T>  // false: not launched, one CTA per particle is as fast
+template <typename T>  // false (32-bit plans): not launched, one CTA per particle is as fast
 bool launch_newton_spread(const Plan &p, const T *c, int B, int batch, const int *n_cand, double *euler,
                           double *score, int *cflags, long long *work, cudaStream_t st, cudaError_t *e);
 template <typename T>

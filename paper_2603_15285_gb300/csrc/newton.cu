@@ -13,7 +13,8 @@
 //   term(-m,-n) = conj(term(m,n))              (real volumes),
 // so one recurrence serves the four orders (m,n), (n,m), (-m,-n), (-n,-m).
 //
-// Work layout: one CTA per particle holds all P candidates.  A warp is split
+// Work layout (32-bit plans that fill the SMs, and the cost-sorted queue; others are
+// spread further, newton_spread.cu): one CTA per particle holds all P candidates.  A warp is split
 // into sub-slots of `cpw` lanes (cpw = P rounded up to a power of two); lane
 // p of a sub-slot follows candidate p.  A sub-slot walks partner groups (the
 // two order pairs (m, n), (m, n+1) of one m, stored interleaved), and each

@@ -18,13 +18,16 @@
 //   soft_grid.cu          grids too large for shared memory, and those only
 //                         k_soft_stream would hold when the caller passes a
 //                         grid: written to memory, then searched;
-//   k_soft_stream, k_soft_chunk
-//                         one CTA per particle, the grid kept on chip
-//                         (streamed by beta slice, or in passes of beta
-//                         slices with a ring of two neighbour slices);
+//   k_soft_stream         one CTA per particle, the grid kept on chip,
+//                         streamed by beta slice;
+//   k_soft_chunk          on chip in passes of beta slices with a ring of two
+//                         neighbour slices, a particle on one CTA or its
+//                         passes over a cluster;
 //   k_soft_warps          the chunked passes with a warp per beta slice;
 //   k_soft_tile           the chunked passes register-tiled for L0 = 8,
-//                         K = 2 in 32-bit plans (the bench configuration).
+//                         K = 2 in 32-bit plans (the bench configuration);
+//   k_soft_split          the same with a particle's passes over a cluster of
+//                         three or nine CTAs, for small batches.
 #include <algorithm>
 #include <float.h>
 #include <limits.h>
@@ -247,10 +250,6 @@ k_soft_stream(const T *__restrict__ c, long nc, int L0, int ns, const int *__res
   if (tid == 0) n_cand_out[b] = kept;
 }
 
-// Chunked streaming variant: each pass computes up to KB+1 new beta slices at
-// once (three phases over all of them) into a ring of KB+2 slices, then tests
-// the local maxima of KB slices and merges them, so each barrier separates
-// KB times more independent work than the one-slice version.
 // The best-P lists of a cluster's CTAs (sorted; the counters' second entry: their
 // length) merged into the first one's, by its first warp.  The order is total, so the
 // split leaves no trace.
@@ -292,6 +291,12 @@ __device__ __forceinline__ typename Vec4<T>::type ld4(const T *p) {
   return *reinterpret_cast<const typename Vec4<T>::type *>(p);
 }
 
+// Chunked streaming variant: each pass computes up to KB+1 new beta slices at
+// once (three phases over all of them) into a ring of KB+2 slices, then tests
+// the local maxima of KB slices and merges them, so each barrier separates
+// KB times more independent work than the one-slice version.
+// CL > 1: the passes of a particle are shared by a cluster of CL CTAs; the first merges
+// the others' best-P lists.
 template <typename T, int KB>
 __global__ void __launch_bounds__(CHUNK_THREADS, sizeof(T) == 8 ? 1 : 2)
 k_soft_chunk(const T *__restrict__ c, long nc, int L0, int ns, const int *__restrict__ pair_base,
