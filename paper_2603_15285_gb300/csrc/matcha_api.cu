@@ -189,16 +189,15 @@ matcha_status matcha_plan_create(const matcha_plan_desc *d, matcha_plan *out) {
   size_t o_rs = add(8 * p->S), o_w = add(8 * p->S), o_x = add(8 * p->nt), o_wj = add(8 * p->nt);
   size_t o_pt = add(rs * p->nlm * p->nt), o_phi = add(rs * 2 * p->np), o_tw = add(rs * 2 * p->ns);
   size_t o_sd = add(rs * p->ns * p->nc0), o_sdT = add(rs * p->ns * p->nc0), o_rc = add(rs * 4 * p->nc), o_K = add(rs * 4 * p->ngroups);
-  size_t o_off = add(4 * p->npairs), o_off0 = add(4 * p->npairs0);
-  size_t o_ptl = add(rs * p->nlm * p->nt), o_leg = add(4 * (size_t)p->nlm);
+  size_t o_ptl = add(rs * p->nlm * p->nt);
   size_t o_dcs = add(rs * 4 * (size_t)p->Qf * p->Mq);
   size_t o_ring = add(rs * 2 * (size_t)p->S * p->nt);
-  size_t o_err = add(sizeof(int));
-  size_t o_fft = add(rs * 2 * (size_t)p->N);
   size_t o_gd = add(rs * GROUP_DESC * (size_t)p->ngroups);
   std::vector<int4> sched;
   p->nrounds = newton_schedule(*p, sched);
-  size_t o_sch = add(sizeof(int4) * sched.size());
+  // the tables made on the host, side by side: one copy (each synchronises, about 8 us)
+  size_t o_err = add(sizeof(int)), o_fft = add(rs * 2 * (size_t)p->N), o_sch = add(sizeof(int4) * sched.size());
+  size_t o_off = add(4 * p->npairs), o_off0 = add(4 * p->npairs0), o_leg = add(4 * (size_t)p->nlm);
   cudaError_t e = cudaGetDevice(&p->device);
   if (e != cudaSuccess) { delete p; return fail_cuda(e, "cudaGetDevice"); }
   cudaDeviceGetAttribute(&p->sms, cudaDevAttrMultiProcessorCount, p->device);
@@ -227,27 +226,28 @@ matcha_status matcha_plan_create(const matcha_plan_desc *d, matcha_plan *out) {
     while (n % 5 == 0 && np < 16) { p->fft_radix[np++] = 5; n /= 5; }
     p->fft_npass = n == 1 ? np : 0;
   }
-  std::vector<double> tw(2 * (size_t)p->N);
+  std::vector<char> host(sz - o_err);  // the status word and the tables after it
+  auto at = [&](size_t o) { return host.data() + (o - o_err); };
   for (int j = 0; j < p->N; ++j) {
-    tw[2 * j] = cos(2.0 * M_PI * j / p->N);
-    tw[2 * j + 1] = -sin(2.0 * M_PI * j / p->N);
+    const double c = cos(2.0 * M_PI * j / p->N), sn = -sin(2.0 * M_PI * j / p->N);
+    if (p->fp64) {
+      ((double *)at(o_fft))[2 * j] = c;
+      ((double *)at(o_fft))[2 * j + 1] = sn;
+    } else {
+      ((float *)at(o_fft))[2 * j] = (float)c;
+      ((float *)at(o_fft))[2 * j + 1] = (float)sn;
+    }
   }
-  std::vector<float> twf(tw.begin(), tw.end());
-  e = cudaMemset(p->dev_err, 0, sizeof(int));
-  if (e == cudaSuccess)
-    e = cudaMemcpy(p->fft_tw, p->fp64 ? (const void *)tw.data() : (const void *)twf.data(),
-                   rs * 2 * (size_t)p->N, cudaMemcpyHostToDevice);
-  if (e == cudaSuccess)
-    e = cudaMemcpy(p->sched, sched.data(), sizeof(int4) * sched.size(), cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMemcpy(p->pair_base, base.data(), 4 * p->npairs, cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMemcpy(p->pair_off0, off0.data(), 4 * p->npairs0, cudaMemcpyHostToDevice);
+  memcpy(at(o_sch), sched.data(), sizeof(int4) * sched.size());
+  memcpy(at(o_off), base.data(), 4 * p->npairs);
+  memcpy(at(o_off0), off0.data(), 4 * p->npairs0);
   {  // Legendre items: m ascending, then the parity of l + m, then l
-    std::vector<int> leg;
+    int *leg = (int *)at(o_leg);
     for (int m = 0; m <= p->LJ; ++m)
       for (int par = 0; par < 2; ++par)
-        for (int l = m + par; l <= p->LJ; l += 2) leg.push_back((l << 16) | m);
-    if (e == cudaSuccess) e = cudaMemcpy(p->leg_lm, leg.data(), 4 * leg.size(), cudaMemcpyHostToDevice);
+        for (int l = m + par; l <= p->LJ; l += 2) *leg++ = (l << 16) | m;
   }
+  e = cudaMemcpy(b + o_err, host.data(), host.size(), cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = build_tables(*p, 0);
   if (e != cudaSuccess) {
     cudaFree(p->base);
