@@ -288,7 +288,8 @@ def kernel_roofline(w, B, prec, stage_ms, alu_peak, m):
         out["contraction"] = {"kernel": "k_correlate_tc", "bound": "tensor", "unit": "TFLOP/s",
                               "peak": tpk, "peak_source": src}
     else:
-        out["contraction"] = {"kernel": "k_correlate_deg", "bound": "alu", "unit": "TFLOP/s",
+        out["contraction"] = {"kernel": "k_correlate_deg" if prec == m.FP64 else "k_correlate_rec",
+                              "bound": "alu", "unit": "TFLOP/s",
                               "peak": alu_peak, "peak_source": "the roofline's ALU peak"}
     c = out["contraction"]
     c["achieved"] = flops / (stage_ms["correlate"] * 1e-3) / 1e12
@@ -785,13 +786,13 @@ def main():
                flags=torch.empty((B,), dtype=torch.int32, device="cuda"))
     H = plan.handle
     stages = ["analyze", "correlate", "soft", "newton", "select"]
-    # Kernels of one matcha_align step: per part of the batch k_analyze2 x2
-    # (particles, templates), the contraction, k_soft_tile (grid and top-P
+    # Kernels of one matcha_align step: per part of the batch k_analyze2
+    # (particles and templates), the contraction, k_soft_tile (grid and top-P
     # fused), k_newton, k_final_select; from 256 particles on the batch runs as
-    # min(4, B / 128) concurrent parts (a shared template is analysed once).
+    # min(4, B / 128) concurrent parts (a shared template is analysed before them).
     n_parts = 1 if B < 256 else min(4, B // 128)  # (batch64's SOFFT is fused)
     shared = temps.shape[0] != B
-    KERNELS_PER_STEP = n_parts * (5 if shared else 6) + (1 if shared else 0)
+    KERNELS_PER_STEP = n_parts * 5 + (1 if shared and n_parts > 1 else 0)
 
     def step(ev=None):
         def mark(i):
